@@ -420,10 +420,14 @@ plhr_status plhr_tharm_extract_noalloc(int m, int kp, int nv, const double* Gzz,
  * tensor-core form computes the full U^T Q.  Block b
  * has n rows, element (i, j) at Z[b][i * ldz[b] + j] (host arrays of device
  * pointers and leading dimensions).  Forms:
- *   PLHR_GRAM_F64     FP64 blocks, FP64 products and sums;
+ *   PLHR_GRAM_F64     FP64 blocks, FP64-class products and sums: six 9-bit
+ *                     slices per value and exact integer sums on the tensor
+ *                     cores, errors about 2^-51 |x| |y| (FP64 multiply-adds
+ *                     when a column holds Inf or NaN);
  *   PLHR_GRAM_F32     FP32 blocks, FP32 products on the FP32 pipes, sums
  *                     folded into double-FP32 every 32 rows;
- *   PLHR_GRAM_DW      FP64 blocks, double-word (hi + lo FP32) arithmetic;
+ *   PLHR_GRAM_DW      FP64 blocks, the form of the mixed solve's FP64-storage
+ *                     phase: the same kernel as PLHR_GRAM_F64;
  *   PLHR_GRAM_F32_TC  FP32 blocks on the tensor cores (tcgen05): each value
  *                     split into three BF16 slices, the six slice products of
  *                     order <= 2 accumulated in FP32 in tensor memory, folded

@@ -77,6 +77,13 @@ cudaError_t multi_gram_b(int64_t n, int nb, const Blk<const double>* Z, const Bl
                          const Blk<const double>* Q, const Blk<const double>* BZ, double sigma,
                          const double* colscale, double* partial, double* out, cudaStream_t s);
 
+// The tensor-core Gram of gram_fx.cu (B = I): *grid CTAs write partial sums
+// (3 m^2 each) and, behind them, one int each in *flags: non-zero when the
+// Grams have to be formed by the plain FP64 kernel instead.
+cudaError_t gram_fx_launch(int64_t n, int nb, const Blk<const double>* Z, const Blk<const double>* AZ,
+                           const Blk<const double>* Q, double sigma, const double* colscale, double* partial,
+                           int* grid, int** flags, cudaStream_t s);
+
 // o1 = AX - BX diag(lam) and o2 = AX - sig BX (each optional), n x nc
 cudaError_t shift_combine(int64_t n, int nc, const double* AX, int64_t ldax, const double* BX, int64_t ldbx,
                           const double* lam, double* o1, int64_t ld1, double sig, double* o2, int64_t ld2,
@@ -102,12 +109,9 @@ cudaError_t gather_columns(int64_t n, const double* X, int64_t ldx, const int* i
 cudaError_t column_dots(int64_t n, int kc, const double* X, int64_t ldx, const double* Y, int64_t ldy,
                         double* partial, double* out, cudaStream_t s);
 
-// Double-word forms of multi_gram and block_update (same arguments and
-// results; inputs rounded once to hi + lo FP32 pairs, products and sums in
-// double-word arithmetic on the FP32 pipes; partial: sm_count() * 3 m^2).
-cudaError_t multi_gram_dw(int64_t n, int nb, const Blk<const double>* Z, const Blk<const double>* AZ,
-                          const Blk<const double>* Q, double sigma, const double* colscale, double* partial,
-                          double* out, cudaStream_t s);
+// Double-word form of block_update (same arguments and results; inputs rounded
+// once to hi + lo FP32 pairs, products and sums in double-word arithmetic on
+// the FP32 pipes).
 cudaError_t block_update_dw(int64_t n, int nb, const Blk<const double>* F, int kp, const double* Cp, const double* Cvv,
                             double* Vout, int64_t ldvo, double* Pout, int64_t ldpo, cudaStream_t s);
 

@@ -57,12 +57,9 @@ plhr_status plhr_gram(int form, int64_t n, int nb, const int* ncols, const void*
             ab[b] = {static_cast<const double*>(AZ[b]), ldaz[b], ncols[b]};
             if (Q) qb[b] = {static_cast<const double*>(Q[b]), ldq[b], ncols[b]};
         }
-        if (form == PLHR_GRAM_F64)
-            PLHR_TRY_CUDA(multi_gram(n, nb, zb.data(), ab.data(), Q ? qb.data() : nullptr, sigma, colscale, partial,
-                                     out, s));
-        else
-            PLHR_TRY_CUDA(multi_gram_dw(n, nb, zb.data(), ab.data(), Q ? qb.data() : nullptr, sigma, colscale,
-                                        partial, out, s));
+        // both forms are the exact-slice tensor-core Gram
+        PLHR_TRY_CUDA(multi_gram(n, nb, zb.data(), ab.data(), Q ? qb.data() : nullptr, sigma, colscale, partial, out,
+                                 s));
     } else {
         std::vector<BlkMx> zb(nb), ab(nb), qb(nb);
         for (int b = 0; b < nb; ++b) {

@@ -223,7 +223,7 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
     // FP32 blocks of the mixed form: W, A W, [S | Q_W], its input, A S, A S - sigma S,
     // Q_S, P, A P, Q_P, Q_V
     bool mx = opt.precision == PLHR_PRECISION_MIXED;
-    // FP64 phase of the mixed form: V-cycle, Gram and update in double-word
+    // FP64 phase of the mixed form: V-cycle and update in double-word
     // arithmetic on the FP64 blocks (FP64-class accuracy on the FP32 pipes)
     const bool dwf = opt.precision == PLHR_PRECISION_MIXED;
     // thq: T-harmonic images Q = T(A - sigma B)Z are formed (T given and the
@@ -817,11 +817,8 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
             da.xi = xi; da.out_int = dstat + 3; da.clk = nullptr;
             {
                 PhaseScope ps(PH_GRAM, s, gram_flops(n, m), 8.0 * n * m * ((thq ? 3 : 2) + (hasB ? 1 : 0)));
-                if (dwf)
-                    PLHR_TRY_CUDA(multi_gram_dw(n, nb, zb, ab, thq ? qb : nullptr, sigma, colscale, gpart, grams, s));
-                else
-                    PLHR_TRY_CUDA(multi_gram_b(n, nb, zb, ab, thq ? qb : nullptr, hasB ? bzb : nullptr, sigma, colscale,
-                                               gpart, grams, s));
+                PLHR_TRY_CUDA(multi_gram_b(n, nb, zb, ab, thq ? qb : nullptr, hasB ? bzb : nullptr, sigma, colscale,
+                                           gpart, grams, s));
             }
             // ---------------------------------------- projected T-harmonic problem, selection (steps 7-10)
             {
