@@ -146,20 +146,50 @@ def _check(status, where):
         raise PlhrError(status, where)
 
 
+_torch = None
+
+
+def _torch_module():
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
 def _stream_ptr(stream):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without a Stream object around it (2 us less
+    # per call; torch.cuda.current_stream() is built on the same function)
+    torch = _torch_module()
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check_block(X, n, name):
-    import torch
+    """The row stride of X, a 2-D row-major float64 CUDA tensor with n rows."""
+    torch = _torch_module()
     if not isinstance(X, torch.Tensor) or not X.is_cuda or X.dtype != torch.float64 or X.dim() != 2:
         raise ValueError("%s must be a 2-D float64 CUDA tensor" % name)
-    if X.shape[0] != n:
-        raise ValueError("%s has %d rows, operator has %d" % (name, X.shape[0], n))
-    if X.stride(1) != 1 or (X.shape[0] > 1 and X.stride(0) < X.shape[1]):
+    rows, cols = X.shape
+    if rows != n:
+        raise ValueError("%s has %d rows, operator has %d" % (name, rows, n))
+    ld, one = X.stride()
+    if one != 1 or (rows > 1 and ld < cols):
         raise ValueError("%s must be row-major with unit column stride" % name)
+    return ld
+
+
+def _apply_block(fn, where, handle, n, X, out, stream, name):
+    """out = T X through the C function fn(handle, cols, X, ldx, out, ldout, stream)."""
+    ldx = _check_block(X, n, name)
+    if out is None:
+        out = _torch.empty_like(X)
+    ldo = _check_block(out, n, "out")
+    st = fn(handle, X.shape[1], X.data_ptr(), ldx, out.data_ptr(), ldo, _stream_ptr(stream))
+    if st != PLHR_OK:
+        raise PlhrError(st, where)
+    return out
 
 
 class Operator:
@@ -167,6 +197,7 @@ class Operator:
 
     def __init__(self, handle, dims, h, scale):
         self._h = handle
+        self.n = int(load_library().plhr_op_size(handle))
         self.dims = tuple(dims)
         self.h = h
         self.scale = scale
@@ -265,20 +296,8 @@ class Operator:
         op._potential = pot
         return op
 
-    @property
-    def n(self):
-        return int(load_library().plhr_op_size(self._h))
-
     def apply(self, X, out=None, stream=None):
-        import torch
-        _check_block(X, self.n, "X")
-        if out is None:
-            out = torch.empty_like(X)
-        _check_block(out, self.n, "out")
-        _check(load_library().plhr_op_apply(self._h, X.shape[1], ctypes.c_void_p(X.data_ptr()), X.stride(0),
-                                            ctypes.c_void_p(out.data_ptr()), out.stride(0), _stream_ptr(stream)),
-               "plhr_op_apply")
-        return out
+        return _apply_block(load_library().plhr_op_apply, "plhr_op_apply", self._h, self.n, X, out, stream, "X")
 
     def apply_c128(self, X, out=None, stream=None):
         """Y = op X for a complex128 CUDA block (n x ncols, row-major)."""
@@ -329,27 +348,12 @@ class AVMG:
         self.sigma = sigma
 
     def apply(self, R, out=None, stream=None):
-        import torch
-        _check_block(R, self.n, "R")
-        if out is None:
-            out = torch.empty_like(R)
-        _check_block(out, self.n, "out")
-        _check(load_library().plhr_prec_apply(self._h, R.shape[1], ctypes.c_void_p(R.data_ptr()), R.stride(0),
-                                              ctypes.c_void_p(out.data_ptr()), out.stride(0), _stream_ptr(stream)),
-               "plhr_prec_apply")
-        return out
+        return _apply_block(load_library().plhr_prec_apply, "plhr_prec_apply", self._h, self.n, R, out, stream, "R")
 
     def apply_dw(self, R, out=None, stream=None):
         """The same V-cycle in double-word arithmetic on float64 CUDA blocks."""
-        import torch
-        _check_block(R, self.n, "R")
-        if out is None:
-            out = torch.empty_like(R)
-        _check_block(out, self.n, "out")
-        _check(load_library().plhr_prec_apply_dw(self._h, R.shape[1], ctypes.c_void_p(R.data_ptr()), R.stride(0),
-                                                 ctypes.c_void_p(out.data_ptr()), out.stride(0), _stream_ptr(stream)),
-               "plhr_prec_apply_dw")
-        return out
+        return _apply_block(load_library().plhr_prec_apply_dw, "plhr_prec_apply_dw", self._h, self.n, R, out, stream,
+                            "R")
 
     def apply_f32(self, R, out=None, stream=None):
         """The same V-cycle in FP32 (the form the mixed-precision solve uses)
@@ -372,15 +376,7 @@ class AVMG:
 
 class _PrecBase:
     def apply(self, R, out=None, stream=None):
-        import torch
-        _check_block(R, self.n, "R")
-        if out is None:
-            out = torch.empty_like(R)
-        _check_block(out, self.n, "out")
-        _check(load_library().plhr_prec_apply(self._h, R.shape[1], ctypes.c_void_p(R.data_ptr()), R.stride(0),
-                                              ctypes.c_void_p(out.data_ptr()), out.stride(0), _stream_ptr(stream)),
-               "plhr_prec_apply")
-        return out
+        return _apply_block(load_library().plhr_prec_apply, "plhr_prec_apply", self._h, self.n, R, out, stream, "R")
 
     def __del__(self):
         if getattr(self, "_h", None) and _lib is not None:
@@ -460,15 +456,7 @@ class TPA:
         self.energy = lib.plhr_prec_tpa_energy(out)
 
     def apply(self, R, out=None, stream=None):
-        import torch
-        _check_block(R, self.n, "R")
-        if out is None:
-            out = torch.empty_like(R)
-        _check_block(out, self.n, "out")
-        _check(load_library().plhr_prec_apply(self._h, R.shape[1], ctypes.c_void_p(R.data_ptr()), R.stride(0),
-                                              ctypes.c_void_p(out.data_ptr()), out.stride(0), _stream_ptr(stream)),
-               "plhr_prec_apply")
-        return out
+        return _apply_block(load_library().plhr_prec_apply, "plhr_prec_apply", self._h, self.n, R, out, stream, "R")
 
     def __del__(self):
         if getattr(self, "_h", None) and _lib is not None:

@@ -135,14 +135,14 @@ extern "C" plhr_status plhr_eigvec_adjoint(const plhr_op* A, plhr_prec* T, int k
     // device workspace: 9 n x k blocks, the k x k cross matrix and partials
     double* ws = nullptr;
     const int64_t need = 9 * nk + k * k + (int64_t)cross_blocks * k * k + (int64_t)res_blocks * 2 * k + 4 * kMaxK;
-    if (cudaMallocAsync(&ws, sizeof(double) * need, s) != cudaSuccess) {
+    if (ws_alloc(reinterpret_cast<void**>(&ws), sizeof(double) * need, s) != cudaSuccess) {
         set_error("plhr_eigvec_adjoint: device allocation failed");
         return PLHR_ENOMEM;
     }
     struct Free {
         double* p;
         cudaStream_t s;
-        ~Free() { cudaStreamSynchronize(s); cudaFree(p); }
+        ~Free() { ws_free(p, s); }
     } fr{ws, s};
     double* q = ws;
     double *x = q; q += nk;

@@ -1,8 +1,10 @@
 // C ABI: error state, stencil operators, the AV-MG preconditioner object.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "plhr_internal.h"
@@ -33,6 +35,59 @@ int sm_count() {
             cached = 132;
     }
     return cached;
+}
+
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
+std::atomic<int> g_live{0};
+
+// the current device's pool, created on its first use; nullptr when there is none
+cudaMemPool_t pool_of_device() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps pr{};
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        unsigned long long keep = kPoolKeep;
+        if (cudaMemPoolCreate(&pool, &pr) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        g_pool[dev] = pool;
+    }
+    return g_pool[dev];
+}
+}  // namespace
+
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s) {
+    cudaMemPool_t pool = pool_of_device();
+    if (!pool) return cudaMallocAsync(p, bytes, s);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+}
+
+void ws_free(void* p, cudaStream_t s) {
+    if (p) cudaFreeAsync(p, s);
+}
+
+LiveObject::LiveObject() { g_live.fetch_add(1); }
+LiveObject::~LiveObject() {
+    if (g_live.fetch_sub(1) != 1) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (cudaMemPool_t pool : g_pool)
+        if (pool) cudaMemPoolTrimTo(pool, 0);
 }
 
 }  // namespace plhr

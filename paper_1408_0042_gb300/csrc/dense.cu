@@ -1373,12 +1373,12 @@ extern "C" plhr_status plhr_tharm_extract(int m, int kp, int nv, const double* G
     }
     cudaStream_t s = (cudaStream_t)stream;
     double* work = nullptr;
-    PLHR_TRY_CUDA(cudaMallocAsync(&work, sizeof(double) * dense_work_doubles(), s));
+    PLHR_TRY_CUDA(ws_alloc(reinterpret_cast<void**>(&work), sizeof(double) * dense_work_doubles(), s));
     DenseArgs a;
     a.m = m; a.kp = kp; a.nv = nv; a.Gzz = Gzz; a.Guq = Guq; a.Gqz = Gqz; a.colscale = colscale; a.work = work;
     a.Cp = Cp; a.Cvv = Cvv; a.tags = tags; a.tag_partner = partner; a.xi = xi; a.out_int = status; a.clk = clk;
     cudaError_t e = dense_extract(a, s);
-    cudaFreeAsync(work, s);
+    ws_free(work, s);
     PLHR_TRY_CUDA(e);
     return PLHR_OK;
 }

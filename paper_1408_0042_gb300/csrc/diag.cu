@@ -40,16 +40,16 @@ plhr_status plhr_gram(int form, int64_t n, int nb, const int* ncols, const void*
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int blocks = std::max(std::max(reduce_blocks(), gram_mx_blocks()), std::max(gram_tc_blocks(), sm_count()));
+    // partial sums, and behind them the tensor-core form's time-out flag
     double* partial = nullptr;
-    int* err = nullptr;
-    PLHR_TRY_CUDA(cudaMallocAsync(&partial, sizeof(double) * (size_t)blocks * 3 * m * m, s));
+    const size_t doubles = (size_t)blocks * 3 * m * m;
+    PLHR_TRY_CUDA(ws_alloc(reinterpret_cast<void**>(&partial), sizeof(double) * (doubles + 1), s));
     struct Free {
-        void* p; void* q; cudaStream_t s;
-        ~Free() { cudaStreamSynchronize(s); if (p) cudaFree(p); if (q) cudaFree(q); }
-    } fr{partial, nullptr, s};
-    PLHR_TRY_CUDA(cudaMallocAsync(&err, sizeof(int), s));
-    fr.q = err;
-    PLHR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+        void* p; cudaStream_t s;
+        ~Free() { ws_free(p, s); }
+    } fr{partial, s};
+    int* err = reinterpret_cast<int*>(partial + doubles);
+    if (form == PLHR_GRAM_F32_TC) PLHR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     if (form == PLHR_GRAM_F64 || form == PLHR_GRAM_DW) {
         std::vector<Blk<const double>> zb(nb), ab(nb), qb(nb);
         for (int b = 0; b < nb; ++b) {
@@ -75,7 +75,8 @@ plhr_status plhr_gram(int form, int64_t n, int nb, const int* ncols, const void*
                                         partial, out, err, s));
     }
     int herr = 0;
-    PLHR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    if (form == PLHR_GRAM_F32_TC)
+        PLHR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     PLHR_TRY_CUDA(cudaStreamSynchronize(s));
     if (herr) {
         set_error("plhr_gram: a tensor-core completion wait timed out");

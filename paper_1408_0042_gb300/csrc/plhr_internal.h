@@ -84,6 +84,22 @@ inline int grid_size_for(int64_t work, int threads, int max_blocks) {
 
 int sm_count();
 
+// Short-lived device workspace (stream-ordered, any thread) from a memory pool
+// of the library's own: freed blocks stay in the pool up to kPoolKeep bytes
+// per device, so that a call does not map and unmap device memory each time
+// (about 100 us per allocation).  The pool gives what it keeps back to the
+// device when the last operator or preconditioner is destroyed, and when an
+// allocation fails (which is then tried again).
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
+void ws_free(void* p, cudaStream_t s);
+// counts the library's live objects
+struct LiveObject {
+    LiveObject();
+    ~LiveObject();
+    LiveObject(const LiveObject&) = delete;
+};
+
 // Kernel launches issued by the library (all entry points, process-wide).
 void count_launches(int n);
 
@@ -239,12 +255,14 @@ int64_t mg_workspace_dw(const MGHierarchy& H, int nc);
 }  // namespace plhr
 
 struct plhr_op {
+    plhr::LiveObject live;
     int kind;
     plhr::Grid g;
     plhr::CsrData csr;   // owned arrays of a CSR operator (g.csr points here)
 };
 
 struct plhr_prec {
+    plhr::LiveObject live;
     int kind = plhr::PREC_AVMG;
     plhr::MGHierarchy H;          // PREC_AVMG
     plhr::SpecPrec sp;            // PREC_TPA
