@@ -332,7 +332,7 @@ cudaError_t multi_gram_b(int64_t n, int nb, const Blk<const double>* Z, const Bl
     int* flags = nullptr;
     if (!BZ) {
         // B = I: exact slices on the tensor cores at every n and m (262,144 rows,
-        // m = 36: 276 us against 2.36 ms); k_gram then only works on columns with Inf
+        // m = 36: 302 us against 2.36 ms); k_gram then only works on columns with Inf
         // or NaN.  With a B family it is the only form.
         cudaError_t e = gram_fx_launch(n, nb, Z, AZ, Q, sigma, colscale, partial, &blocks, &flags, s);
         if (e != cudaSuccess) return e;

@@ -31,10 +31,9 @@
 // multiply-adds give 5.7e-16 to 1.5e-15 and double-word ones 5e-15 to 5e-13.
 //
 // Exponents.  E is kept per column and CTA: the largest exponent met so far
-// plus one (plus two in long runs).  When a value exceeds it, the pending period
-// is folded, the integers are shifted to the new exponents and the CTA goes on
-// (each CTA starts with its middle rows, which on a grid are rarely the
-// smallest).  So the precision is relative to the columns' norms (what the
+// plus one (plus two in long runs), from 32 rows spread over the CTA's share on.
+// When a value exceeds it, the pending period is folded, the integers are
+// shifted to the new exponents and the CTA goes on.  So the precision is relative to the columns' norms (what the
 // Cholesky factorisation of a Gram matrix needs), not to each pair of entries.
 // A column holding Inf or NaN and a wait that times out set the CTA's flag: the
 // plain FP64 kernel, which is launched behind this one and returns at once
@@ -57,9 +56,9 @@
 // integer and FP32 instructions per value, is what binds: 4.6k of 9k cycles
 // per step, the rest loads, the barrier and the read-back.
 //
-// Measured on GB300: m = 36, 262,144 rows 276 us (FP64 multiply-adds 2.36 ms,
-// bound by the FP64 pipe); m = 64, 2,097,152 rows 2.36 ms (double-word
-// multiply-adds on the FP32 pipes 9.45 ms).
+// Measured on GB300 on trial bases of a Laplacian: m = 36, 262,144 rows 302 us
+// (FP64 multiply-adds 2.36 ms, bound by the FP64 pipe); m = 64, 2,097,152 rows
+// 2.47 ms (double-word multiply-adds on the FP32 pipes 9.45 ms).
 #include "blockops.h"
 #include "tc.h"
 
@@ -457,14 +456,44 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                 mq = max(mq, exp_field(qv[i]));
             }
         };
+        // raise the exponents of the warp's columns to the loaded values (Inf and NaN
+        // set the flag and leave them alone); whether this thread's had to
+        auto raise = [&]() -> bool {
+            const bool up = mz >= ez || mu >= eu || mq >= eq;
+            if (!__any_sync(0xffffffffu, up)) return false;
+            if (mz == 0x7ff || mu == 0x7ff || mq == 0x7ff) bad = true;
+            auto one = [&](int& e, int mx, int at_col) {
+                int x = mx >= e && mx != 0x7ff ? mx + room : e;
+                for (int o = 4; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+                e = x;
+                if ((lane & 7) == 0 && conv) S.en[at_col] = x;
+            };
+            one(ez, mz, j);
+            one(eq, mq, mp + j);
+            one(eu, mu, 2 * mp + j);
+            return up;
+        };
         bool pending = false, first = true;    // accumulators hold products not yet added / nothing written yet
-        if (nst > 0) {
-            start_of(0);
+        auto load = [&]() {
             if (conv) {
                 load4(0, z);
                 load4(1, a);
                 if (has_q) load4(2, qv);
             }
+        };
+        if (nst > 16) {
+            // 32 rows spread over the CTA's share set the first exponents: smooth columns
+            // then hardly ever outgrow them (m = 36, 262,144 rows: 370 -> 302 us)
+            start_of((int)((int64_t)(lane & 7) * nst / 8));
+            load();
+            if (conv) prepare();
+            if (convw) raise();
+            conv_sync();
+            if (tid < 3 * mp) S.e[tid] = S.en[tid];
+        }
+        if (nst > 0) {
+            start_of(0);
+            load();
         }
         // one step more than there is: it drains the last period and writes the sums
         for (int st = 0; st <= nst; ++st) {
@@ -472,22 +501,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
             bool grow = false, w = true;
             if (!last) {
                 if (conv) prepare();
-                if (convw) {
-                    grow = mz >= ez || mu >= eu || mq >= eq;
-                    if (__any_sync(0xffffffffu, grow)) {
-                        // Inf and NaN set the flag and leave the exponents alone
-                        if (mz == 0x7ff || mu == 0x7ff || mq == 0x7ff) bad = true;
-                        auto raise = [&](int& e, int mx, int at_col) {
-                            int x = mx >= e && mx != 0x7ff ? mx + room : e;
-                            for (int o = 4; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
-                            e = x;
-                            if ((lane & 7) == 0 && conv) S.en[at_col] = x;
-                        };
-                        raise(ez, mz, j);
-                        raise(eq, mq, mp + j);
-                        raise(eu, mu, 2 * mp + j);
-                    }
-                }
+                if (convw) grow = raise();
                 // the MMAs of two steps ago have read this panel
                 if (st >= 2) w = tc::mbar_wait(&S.done[st & 1], (uint32_t)(((st >> 1) - 1) & 1), kFxWait);
                 unsigned char* pan = smem + (st & 1) * panel_of(mp);
