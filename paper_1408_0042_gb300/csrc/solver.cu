@@ -55,6 +55,7 @@ struct HostStatus {
     int dense[3];
     int rr_ok;
     int pad;
+    int rr_ok2, pad2;
 };
 
 // flops of one multi-Gram pass over an n x m trial basis: Z^T Z and U^T Q
@@ -448,6 +449,27 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
         return PLHR_OK;
     };
 
+    // The Ritz vectors of the final Rayleigh-Ritz once more, on their own Grams:
+    // Cholesky of an ill-conditioned V^T B V leaves them orthonormal only to
+    // rounding times its condition (4e-12 when two guard columns had nearly
+    // merged), a second pass to rounding.  Rc (and with images QV) is replaced,
+    // A Rc and B Rc are formed anew; dots is left holding ones.
+    auto polish_ritz = [&](bool images) -> plhr_status {
+        std::vector<double> ones(kp, 1.0);
+        PLHR_TRY_CUDA(cudaMemcpyAsync(dots, ones.data(), sizeof(double) * kp, cudaMemcpyHostToDevice, s));
+        PLHR_TRY_CUDA(lap_axpby(g, kp, Rc, kp, AW, kp, 1.0, 0.0, s));
+        if (hasB) PLHR_TRY_CUDA(lap_axpby(B->g, kp, Rc, kp, X3, kp, 1.0, 0.0, s));
+        Blk<const double> zb[1] = {{Rc, kp, kp}}, ab[1] = {{AW, kp, kp}}, bzb[1] = {{X3, kp, kp}};
+        PLHR_TRY_CUDA(multi_gram_b(n, 1, zb, ab, zb, hasB ? bzb : nullptr, 0.0, dots, gpart, grams, s));
+        PLHR_TRY_CUDA(dense_rr(kp, grams + kp * kp, grams, sigma, dots, Crr, theta, dstat + 8, s));
+        PLHR_TRY_CUDA(block_times_small(n, Rc, kp, kp, Crr, kp, Rc, kp, s));
+        if (images) PLHR_TRY_CUDA(block_times_small(n, QV, kp, kp, Crr, kp, QV, kp, s));
+        PLHR_TRY_CUDA(lap_axpby(g, kp, Rc, kp, AW, kp, 1.0, 0.0, s));
+        if (hasB) PLHR_TRY_CUDA(lap_axpby(B->g, kp, Rc, kp, X3, kp, 1.0, 0.0, s));
+        PLHR_TRY_CUDA(cudaMemcpyAsync(&hs->rr_ok2, dstat + 8, sizeof(int), cudaMemcpyDeviceToHost, s));
+        return PLHR_OK;
+    };
+
     // end of the FP32 form: P to FP64, then A V, A P, T(A V - sigma V) and
     // T(A P - sigma P) explicitly in FP64
     // ord: host column order by distance to sigma (the first k are kept)
@@ -568,12 +590,8 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
             }
             PLHR_TRY_CUDA(dense_rr(kp, grams + kp * kp, grams, sigma, scale, Crr, theta, dstat + 6, s));
             PLHR_TRY_CUDA(block_times_small(n, V, kp, kp, Crr, kp, Rc, kp, s));   // all Ritz vectors
-            PLHR_TRY_CUDA(lap_axpby(g, kp, Rc, kp, AW, kp, 1.0, 0.0, s));
-            if (hasB) PLHR_TRY_CUDA(lap_axpby(B->g, kp, Rc, kp, X3, kp, 1.0, 0.0, s));
-            {
-                std::vector<double> ones(kp, 1.0);
-                PLHR_TRY_CUDA(cudaMemcpyAsync(dots, ones.data(), sizeof(double) * kp, cudaMemcpyHostToDevice, s));
-            }
+            if (!mx && thq) PLHR_TRY_CUDA(block_times_small(n, QV, kp, kp, Crr, kp, QV, kp, s));
+            PLHR_TRY(polish_ritz(!mx && thq));
             PLHR_TRY_CUDA(residual_norms(n, kp, hasB ? X3 : Rc, kp, AW, kp, theta, dots, R, kp, rpart, sums, s));
             sa.lam = theta;
             PLHR_TRY_CUDA(dense_status(sa, s));
@@ -581,7 +599,7 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
             PLHR_TRY_CUDA(cudaMemcpyAsync(h_rel, rel, sizeof(double) * kp, cudaMemcpyDeviceToHost, s));
             PLHR_TRY_CUDA(cudaMemcpyAsync(h_theta, theta, sizeof(double) * kp, cudaMemcpyDeviceToHost, s));
             PLHR_TRY_CUDA(cudaStreamSynchronize(s));
-            if (!hs->rr_ok) {
+            if (!hs->rr_ok || !hs->rr_ok2) {
                 set_error("plhr_solve: final Rayleigh-Ritz failed");
                 result = PLHR_EBREAKDOWN;
                 break;
@@ -596,7 +614,6 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
             PLHR_TRY_CUDA(cudaMemcpyAsync(V, Rc, sizeof(double) * nk, cudaMemcpyDeviceToDevice, s));
             PLHR_TRY_CUDA(cudaMemcpyAsync(AV, AW, sizeof(double) * nk, cudaMemcpyDeviceToDevice, s));
             if (hasB) PLHR_TRY_CUDA(cudaMemcpyAsync(BV, X3, sizeof(double) * nk, cudaMemcpyDeviceToDevice, s));
-            if (!mx && thq) PLHR_TRY_CUDA(block_times_small(n, QV, kp, kp, Crr, kp, QV, kp, s));
             PLHR_TRY_CUDA(cudaMemcpyAsync(lam, theta, sizeof(double) * kp, cudaMemcpyDeviceToDevice, s));
             {
                 std::vector<double> ones(kp, 1.0);
@@ -873,10 +890,7 @@ extern "C" plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sig
             PLHR_TRY_CUDA(multi_gram_b(n, 1, zb, ab, qb, hasB ? bzb : nullptr, 0.0, colscale, gpart, grams, s));
             PLHR_TRY_CUDA(dense_rr(kp, grams + kp * kp, grams, sigma, scale, Crr, theta, dstat + 6, s));
             PLHR_TRY_CUDA(block_times_small(n, V, kp, kp, Crr, kp, Rc, kp, s));
-            PLHR_TRY_CUDA(lap_axpby(g, kp, Rc, kp, AW, kp, 1.0, 0.0, s));
-            if (hasB) PLHR_TRY_CUDA(lap_axpby(B->g, kp, Rc, kp, X3, kp, 1.0, 0.0, s));
-            std::vector<double> ones(kp, 1.0);
-            PLHR_TRY_CUDA(cudaMemcpyAsync(dots, ones.data(), sizeof(double) * kp, cudaMemcpyHostToDevice, s));
+            PLHR_TRY(polish_ritz(false));
             PLHR_TRY_CUDA(residual_norms(n, kp, hasB ? X3 : Rc, kp, AW, kp, theta, dots, R, kp, rpart, sums, s));
             StatusArgs sa;
             sa.kp = kp; sa.k = k; sa.sigma = sigma; sa.tol = tol;
