@@ -17,6 +17,7 @@
 // INV-MG (Appendix A, Algorithm 5; H.indefinite): the same cycle with
 // B_l = L_l - sigma I_l on every level (the shift enters the sweeps and the
 // residual) and the signed coarsest solve S diag(1 / (mu - sigma)) S^T.
+#include "mgcoarse.h"
 #include "plhr_internal.h"
 
 namespace plhr {
@@ -44,18 +45,17 @@ __device__ __forceinline__ void unflat(int64_t row, const G3& g, int64_t& ix, in
     iz = t / g.ny;
 }
 
-// 2d/h^2 u - sum of neighbours / h^2 (scaled by ih2), zero outside the grid
+// Sum of the neighbours of x at xp, zero outside the grid
 template <bool D3>
-__device__ __forceinline__ double lap_pt(const double* __restrict__ xp, int64_t ld, int64_t ix, int64_t iy,
+__device__ __forceinline__ double nb_sum(const double* __restrict__ xp, int64_t ld, int64_t ix, int64_t iy,
                                          int64_t iz, const G3& g) {
-    double s = (D3 ? 6.0 : 4.0) * xp[0];
-    if (ix > 0) s -= xp[-ld];
-    if (ix < g.nx - 1) s -= xp[ld];
-    if (iy > 0) s -= xp[-ld * g.nx];
-    if (iy < g.ny - 1) s -= xp[ld * g.nx];
+    const int64_t sy = ld * g.nx, sz = sy * g.ny;
+    const double x0 = ix > 0 ? xp[-ld] : 0.0, x1 = ix < g.nx - 1 ? xp[ld] : 0.0;
+    const double y0 = iy > 0 ? xp[-sy] : 0.0, y1 = iy < g.ny - 1 ? xp[sy] : 0.0;
+    double s = (x0 + x1) + (y0 + y1);
     if (D3) {
-        if (iz > 0) s -= xp[-ld * g.nx * g.ny];
-        if (iz < g.nz - 1) s -= xp[ld * g.nx * g.ny];
+        const double z0 = iz > 0 ? xp[-sz] : 0.0, z1 = iz < g.nz - 1 ? xp[sz] : 0.0;
+        s += z0 + z1;
     }
     return s;
 }
@@ -64,53 +64,53 @@ __device__ __forceinline__ double lap_pt(const double* __restrict__ xp, int64_t 
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (total);        \
          e += (int64_t)gridDim.x * blockDim.x)
 
-// w_out = w_in + om * (r - (ih2 * L - shift) w_in)    (w_in may be null: w_out = om r);
-// SHIFT = false is the AV-MG sweep (shift 0, the expression without the shift term)
-template <bool D3, bool SHIFT>
-__global__ void __launch_bounds__(kT) k_rich_lap(G3 g, int nc, double ih2, double shift, double om,
-                                                 const double* __restrict__ win, const double* __restrict__ r,
-                                                 int64_t ldr, double* __restrict__ wout, int64_t total) {
-    GRID_LOOP(total) {
-        int64_t row;
-        int c;
-        split_index(e, nc, row, c);
-        double rv = r[row * ldr + c];
-        double v;
-        if (win) {
-            int64_t ix, iy, iz;
-            unflat(row, g, ix, iy, iz);
-            const double* wp = win + row * nc + c;
-            if (SHIFT) v = wp[0] + om * (rv - (ih2 * lap_pt<D3>(wp, nc, ix, iy, iz, g) - shift * wp[0]));
-            else v = wp[0] + om * (rv - ih2 * lap_pt<D3>(wp, nc, ix, iy, iz, g));
-        } else {
-            v = om * rv;
-        }
-        wout[row * nc + c] = v;
-    }
-}
+// The FP64 pipe (1/64 of the FP32 rate) binds these kernels, so each is written
+// in as few FP64 operations as its stencil allows: five additions for the
+// neighbours and one multiply(-add) per coefficient, the coefficients formed on
+// the host.  (64^3 x 16: a sweep 77 -> 69 us; the first two sweeps, one kernel
+// now, 95 -> 61 us.)
 
-// t = ih2 * L x - sig * x
-template <bool D3>
-__global__ void __launch_bounds__(kT) k_shifted(G3 g, int nc, double ih2, double sig, const double* __restrict__ x,
-                                                double* __restrict__ t, int64_t total) {
+// out = cx x + cn sum of x's neighbours (+ cr r when r is given): the sweeps
+// w + om (r - (ih2 L - shift) w), 2 om r - om^2 (ih2 L - shift) r (the first two
+// sweeps from zero in one), the residual r - (ih2 L - shift) w and (ih2 L - sig) x
+template <bool D3, bool R>
+__global__ void __launch_bounds__(kT) k_stencil(G3 g, int nc, double cx, double cn, double cr,
+                                                const double* __restrict__ x, int64_t ldx,
+                                                const double* __restrict__ r, int64_t ldr, double* __restrict__ out,
+                                                int64_t total) {
     GRID_LOOP(total) {
         int64_t row;
         int c;
         split_index(e, nc, row, c);
         int64_t ix, iy, iz;
         unflat(row, g, ix, iy, iz);
-        const double* xp = x + row * nc + c;
-        t[row * nc + c] = ih2 * lap_pt<D3>(xp, nc, ix, iy, iz, g) - sig * xp[0];
+        const double* xp = x + row * ldx + c;
+        const double s = nb_sum<D3>(xp, ldx, ix, iy, iz, g);
+        double v = cn * s;
+        if (R) v = fma(cr, r[row * ldr + c], v);
+        out[row * nc + c] = fma(cx, xp[0], v);
     }
 }
 
-// B w for the polynomial level from t = (L - sig) w:  ((L - sig) t + c^2 w) / (2c)
-// mode 0: w_out = w + om (r - Bw);  mode 1: w_out = r - Bw (residual)
+// w = om r (one sweep from zero)
+__global__ void __launch_bounds__(kT) k_scale(int nc, double om, const double* __restrict__ r, int64_t ldr,
+                                              double* __restrict__ w, int64_t total) {
+    GRID_LOOP(total) {
+        int64_t row;
+        int c;
+        split_index(e, nc, row, c);
+        w[e] = om * r[row * ldr + c];
+    }
+}
+
+// polynomial level, t = (L - sig) w, B w = ((L - sig) t + c^2 w) / (2 c):
+// out = cw w + cr r + ct t + cn sum of t's neighbours is the sweep w + om (r - B w)
+// or the residual r - B w
 template <bool D3>
-__global__ void __launch_bounds__(kT) k_poly_step(G3 g, int nc, double ih2, double sig, double cpar, double om,
-                                                  int mode, const double* __restrict__ w,
-                                                  const double* __restrict__ t, const double* __restrict__ r,
-                                                  int64_t ldr, double* __restrict__ out, int64_t total) {
+__global__ void __launch_bounds__(kT) k_poly_step(G3 g, int nc, double cw, double cr, double ct, double cn,
+                                                  const double* __restrict__ w, const double* __restrict__ t,
+                                                  const double* __restrict__ r, int64_t ldr, double* __restrict__ out,
+                                                  int64_t total) {
     GRID_LOOP(total) {
         int64_t row;
         int c;
@@ -118,113 +118,119 @@ __global__ void __launch_bounds__(kT) k_poly_step(G3 g, int nc, double ih2, doub
         int64_t ix, iy, iz;
         unflat(row, g, ix, iy, iz);
         const double* tp = t + row * nc + c;
-        double tt = ih2 * lap_pt<D3>(tp, nc, ix, iy, iz, g) - sig * tp[0];
-        double wv = w[row * nc + c];
-        double bw = (tt + cpar * cpar * wv) / (2.0 * cpar);
-        double res = r[row * ldr + c] - bw;
-        out[row * nc + c] = mode == 0 ? wv + om * res : res;
+        double v = fma(ct, tp[0], cn * nb_sum<D3>(tp, nc, ix, iy, iz, g));
+        v = fma(cw, w[row * nc + c], v);
+        out[row * nc + c] = fma(cr, r[row * ldr + c], v);
     }
 }
 
-// res = r - (ih2 * L - shift) w  (SHIFT = false: r - ih2 * L w)
-template <bool D3, bool SHIFT>
-__global__ void __launch_bounds__(kT) k_resid_lap(G3 g, int nc, double ih2, double shift, const double* __restrict__ w,
-                                                  const double* __restrict__ r, int64_t ldr,
-                                                  double* __restrict__ out, int64_t total) {
-    GRID_LOOP(total) {
-        int64_t row;
-        int c;
-        split_index(e, nc, row, c);
-        int64_t ix, iy, iz;
-        unflat(row, g, ix, iy, iz);
-        if (SHIFT)
-            out[row * nc + c] = r[row * ldr + c] - (ih2 * lap_pt<D3>(w + row * nc + c, nc, ix, iy, iz, g) -
-                                                    shift * w[row * nc + c]);
-        else
-            out[row * nc + c] = r[row * ldr + c] - ih2 * lap_pt<D3>(w + row * nc + c, nc, ix, iy, iz, g);
-    }
-}
+// Transfers, one segment of a grid line per CTA, separably, with the
+// weights' common power of two taken out: linear prolongation is (3 a + b) / 4
+// per axis (a the coarse cell of the fine point, b the next nearest, zero
+// outside), linear restriction (3 (a + b) + (c + d)) / 8 (a, b the children of
+// the coarse cell, c, d the fine points beside them); constant ones are a and
+// (a + b) / 2.  The y-z part of a segment goes to shared memory, then x.  4.5 and 3.5
+// FP64 operations per fine value instead of the 24 and 25 of a tensor product of
+// weights per point.  (64^3 x 16: restriction 116 -> 58 us, prolongation 174 -> 35 us.)
 
-// 1D cell-centred prolongation weights from coarse cells to fine point f:
-// constant: f -> (f/2, 1);  linear: f -> (f/2, 3/4) and (f/2 -+ 1, 1/4)
-__device__ __forceinline__ int pw1(int lin, int64_t f, int64_t nc_axis, int64_t* idx, double* wt) {
-    int64_t I = f >> 1;
-    idx[0] = I;
-    if (!lin) {
-        wt[0] = 1.0;
-        return 1;
-    }
-    wt[0] = 0.75;
-    int64_t J = (f & 1) ? I + 1 : I - 1;
-    if (J < 0 || J >= nc_axis) return 1;
-    idx[1] = J;
-    wt[1] = 0.25;
-    return 2;
-}
+struct LineCut {
+    int cols;   // columns per CTA (blockIdx.y: first one / cols)
+    int seg;    // coarse points per CTA (blockIdx.z: first one / seg)
+};
 
-// w_fine += P w_coarse
+// w_fine += P w_coarse on fine line blockIdx.x = (y, z)
 template <bool D3>
-__global__ void __launch_bounds__(kT) k_prolong_add(G3 gf, G3 gc, int nc, int lin, const double* __restrict__ wc,
-                                                    double* __restrict__ wf, int64_t total) {
-    GRID_LOOP(total) {
-        int64_t row;
-        int c;
-        split_index(e, nc, row, c);
-        int64_t ix, iy, iz;
-        unflat(row, gf, ix, iy, iz);
-        int64_t xi[2], yi[2], zi[2];
-        double xw[2], yw[2], zw[2];
-        int nxw = pw1(lin, ix, gc.nx, xi, xw);
-        int nyw = pw1(lin, iy, gc.ny, yi, yw);
-        int nzw = D3 ? pw1(lin, iz, gc.nz, zi, zw) : 1;
-        if (!D3) { zi[0] = 0; zw[0] = 1.0; }
-        double s = 0.0;
-        for (int a = 0; a < nzw; ++a)
-            for (int b = 0; b < nyw; ++b)
-                for (int q = 0; q < nxw; ++q)
-                    s += zw[a] * yw[b] * xw[q] * wc[((zi[a] * gc.ny + yi[b]) * gc.nx + xi[q]) * nc + c];
-        wf[row * nc + c] += s;
+__global__ void __launch_bounds__(kT) k_prolong_line(G3 gf, G3 gc, int nc, LineCut k, int lin,
+                                                     const double* __restrict__ wc, double* __restrict__ wf) {
+    extern __shared__ double line_sh[];   // [coarse x0 - 1 ..][column]
+    const int64_t line = blockIdx.x;
+    const int64_t iz = line / gf.ny, iy = line - iz * gf.ny;
+    const int c0 = blockIdx.y * k.cols, cols = min(k.cols, nc - c0);
+    const int x0 = blockIdx.z * k.seg, seg = min(k.seg, (int)gc.nx - x0);
+    const int64_t ya = iy >> 1, yb = (iy & 1) ? ya + 1 : ya - 1;
+    const int64_t za = D3 ? iz >> 1 : 0, zb = (iz & 1) ? za + 1 : za - 1;
+    const bool hy = lin && yb >= 0 && yb < gc.ny, hz = D3 && lin && zb >= 0 && zb < gc.nz;
+    const double* paa = wc + (za * gc.ny + ya) * gc.nx * nc + c0;
+    const double* pab = wc + (za * gc.ny + yb) * gc.nx * nc + c0;
+    const double* pba = wc + (zb * gc.ny + ya) * gc.nx * nc + c0;
+    const double* pbb = wc + (zb * gc.ny + yb) * gc.nx * nc + c0;
+    for (int t = threadIdx.x; t < (seg + 2) * cols; t += kT) {
+        const int q = t / cols, c = t - q * cols;
+        const int x = x0 - 1 + q;
+        double v = 0.0;
+        if (x >= 0 && x < (int)gc.nx) {
+            const int64_t o = (int64_t)x * nc + c;
+            v = paa[o];
+            if (lin) {
+                const double vb = hy ? pab[o] : 0.0;
+                v = fma(3.0, v, vb);
+                if (D3) {
+                    const double wa = hz ? pba[o] : 0.0, wb = hz && hy ? pbb[o] : 0.0;
+                    v = fma(3.0, v, fma(3.0, wa, wb));
+                }
+            }
+        }
+        line_sh[t] = v;
+    }
+    __syncthreads();
+    const double scale = lin ? (D3 ? 0x1p-6 : 0x1p-4) : 1.0;
+    for (int t = threadIdx.x; t < 2 * seg * cols; t += kT) {
+        const int x = t / cols, c = t - x * cols;   // fine point 2 x0 + x
+        const double* u = line_sh + ((x >> 1) + 1) * cols + c;
+        double v = u[0];
+        if (lin) v = fma(3.0, v, (x & 1) ? u[cols] : u[-cols]);
+        double* w = wf + (line * gf.nx + 2 * x0 + x) * nc + c0 + c;
+        *w = fma(scale, v, *w);
     }
 }
 
-// 1D restriction taps R = P^T / 2 per axis: coarse I gathers fine 2I, 2I+1
-// (weight 1/2 each, constant) or additionally 2I-1, 2I+2 (linear: 3/8, 3/8,
-// 1/8, 1/8).
-__device__ __forceinline__ int rw1(int lin, int64_t I, int64_t nf_axis, int64_t* idx, double* wt) {
-    if (!lin) {
-        idx[0] = 2 * I; wt[0] = 0.5;
-        idx[1] = 2 * I + 1; wt[1] = 0.5;
-        return 2;
-    }
-    int n = 0;
-    idx[n] = 2 * I; wt[n++] = 0.375;
-    idx[n] = 2 * I + 1; wt[n++] = 0.375;
-    if (2 * I - 1 >= 0) { idx[n] = 2 * I - 1; wt[n++] = 0.125; }
-    if (2 * I + 2 < nf_axis) { idx[n] = 2 * I + 2; wt[n++] = 0.125; }
-    return n;
-}
-
+// rc = R f on coarse line blockIdx.x = (y, z)
 template <bool D3>
-__global__ void __launch_bounds__(kT) k_restrict(G3 gf, G3 gc, int nc, int lin, const double* __restrict__ f,
-                                                 double* __restrict__ rc, int64_t total) {
-    GRID_LOOP(total) {
-        int64_t row;
-        int c;
-        split_index(e, nc, row, c);
-        int64_t ix, iy, iz;
-        unflat(row, gc, ix, iy, iz);
-        int64_t xi[4], yi[4], zi[4];
-        double xw[4], yw[4], zw[4];
-        int nxw = rw1(lin, ix, gf.nx, xi, xw);
-        int nyw = rw1(lin, iy, gf.ny, yi, yw);
-        int nzw = D3 ? rw1(lin, iz, gf.nz, zi, zw) : 1;
-        if (!D3) { zi[0] = 0; zw[0] = 1.0; }
-        double s = 0.0;
-        for (int a = 0; a < nzw; ++a)
-            for (int b = 0; b < nyw; ++b)
-                for (int q = 0; q < nxw; ++q)
-                    s += zw[a] * yw[b] * xw[q] * f[((zi[a] * gf.ny + yi[b]) * gf.nx + xi[q]) * nc + c];
-        rc[row * nc + c] = s;
+__global__ void __launch_bounds__(kT) k_restrict_line(G3 gf, G3 gc, int nc, LineCut k, int lin,
+                                                      const double* __restrict__ f, double* __restrict__ rc) {
+    extern __shared__ double line_sh[];   // [fine 2 x0 - 1 ..][column]
+    const int64_t line = blockIdx.x;
+    const int64_t iz = line / gc.ny, iy = line - iz * gc.ny;
+    const int c0 = blockIdx.y * k.cols, cols = min(k.cols, nc - c0);
+    const int x0 = blockIdx.z * k.seg, seg = min(k.seg, (int)gc.nx - x0);
+    const int64_t ys = gf.nx * nc, zs = ys * gf.ny;
+    const bool y0 = lin && 2 * iy - 1 >= 0, y3 = lin && 2 * iy + 2 < gf.ny;
+    const bool z0 = D3 && lin && 2 * iz - 1 >= 0, z3 = D3 && lin && 2 * iz + 2 < gf.nz;
+    const double* p0 = f + 2 * iy * ys + (D3 ? 2 * iz * zs : 0) + c0;
+    // the y sum of a fine plane, in eighths (halves when constant)
+    auto ysum = [&](const double* p) {
+        const double a = p[0], b = p[ys];
+        if (!lin) return a + b;
+        const double c = y0 ? p[-ys] : 0.0, d = y3 ? p[2 * ys] : 0.0;
+        return fma(3.0, a + b, c + d);
+    };
+    for (int t = threadIdx.x; t < (2 * seg + 2) * cols; t += kT) {
+        const int q = t / cols, c = t - q * cols;
+        const int x = 2 * x0 - 1 + q;
+        double v = 0.0;
+        if (x >= 0 && x < (int)gf.nx) {
+            const double* p = p0 + (int64_t)x * nc + c;
+            v = ysum(p);
+            if (D3) {
+                const double b = ysum(p + zs);
+                if (!lin) {
+                    v += b;
+                } else {
+                    const double cz = z0 ? ysum(p - zs) : 0.0, d = z3 ? ysum(p + 2 * zs) : 0.0;
+                    v = fma(3.0, v + b, cz + d);
+                }
+            }
+        }
+        line_sh[t] = v;
+    }
+    __syncthreads();
+    const double scale = lin ? (D3 ? 0x1p-9 : 0x1p-6) : (D3 ? 0x1p-3 : 0x1p-2);
+    for (int t = threadIdx.x; t < seg * cols; t += kT) {
+        const int x = t / cols, c = t - x * cols;
+        const double* p = line_sh + (2 * x + 1) * cols + c;
+        double v = p[0] + p[cols];
+        if (lin) v = fma(3.0, v, p[-cols] + p[2 * cols]);
+        rc[(line * gc.nx + x0 + x) * nc + c0 + c] = scale * v;
     }
 }
 
@@ -326,58 +332,56 @@ struct LevelBufs {
     double* wc;    // coarse correction from the next coarser level
 };
 
-cudaError_t rich_sweep(const MGLevel& L, double sigma, int nc, const double* win, const double* r, int64_t ldr,
-                       double* tmp, double* wout, cudaStream_t s) {
+// out = cx x + cn sum of neighbours (+ cr r)
+void launch_stencil(const Grid& g, int nc, double cx, double cn, double cr, const double* x, int64_t ldx,
+                    const double* r, int64_t ldr, double* out, cudaStream_t s) {
+    const int64_t total = g.n() * nc;
+    const G3 G = g3(g);
+    const int nb = nblk(total);
+    if (g.d == 3) {
+        if (r) k_stencil<true, true><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
+        else k_stencil<true, false><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
+    } else {
+        if (r) k_stencil<false, true><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
+        else k_stencil<false, false><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
+    }
+    count_launches(1);
+}
+
+// out = cw w + cr (r - B w), B the level's operator (tmp: scratch of a polynomial level)
+cudaError_t level_step(const MGLevel& L, double sigma, int nc, double cw, double cr, const double* w, const double* r,
+                       int64_t ldr, double* tmp, double* out, cudaStream_t s) {
     const Grid& g = L.g;
-    int64_t total = g.n() * nc;
-    G3 G = g3(g);
-    bool d3 = g.d == 3;
-    const double shift = L.shifted ? sigma : 0.0;
-    if (!L.poly || win == nullptr) {
-        const double* wi = L.poly ? nullptr : win;
-        if (L.shifted) {
-            if (d3) k_rich_lap<true, true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), shift, L.omega, wi, r, ldr, wout, total);
-            else k_rich_lap<false, true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), shift, L.omega, wi, r, ldr, wout, total);
-        } else {
-            if (d3) k_rich_lap<true, false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), 0.0, L.omega, wi, r, ldr, wout, total);
-            else k_rich_lap<false, false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), 0.0, L.omega, wi, r, ldr, wout, total);
-        }
-        count_launches(1);
+    const double ih2 = g.inv_h2(), diag = 2.0 * g.d * ih2;
+    if (!L.poly) {
+        const double shift = L.shifted ? sigma : 0.0;
+        launch_stencil(g, nc, cw - cr * (diag - shift), cr * ih2, cr, w, nc, r, ldr, out, s);
         return cudaGetLastError();
     }
-    if (d3) k_shifted<true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, win, tmp, total);
-    else k_shifted<false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, win, tmp, total);
-    count_launches(1);
-    if (d3) k_poly_step<true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, L.c, L.omega, 0, win, tmp, r, ldr, wout, total);
-    else k_poly_step<false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, L.c, L.omega, 0, win, tmp, r, ldr, wout, total);
+    launch_stencil(g, nc, diag - sigma, -ih2, 0.0, w, nc, nullptr, 0, tmp, s);
+    const double cb = cr / (2.0 * L.c);   // weight of (L - sig) t + c^2 w
+    const int64_t total = g.n() * nc;
+    if (g.d == 3)
+        k_poly_step<true><<<nblk(total), kT, 0, s>>>(g3(g), nc, cw - cb * L.c * L.c, cr, -cb * (diag - sigma), cb * ih2,
+                                                     w, tmp, r, ldr, out, total);
+    else
+        k_poly_step<false><<<nblk(total), kT, 0, s>>>(g3(g), nc, cw - cb * L.c * L.c, cr, -cb * (diag - sigma), cb * ih2,
+                                                      w, tmp, r, ldr, out, total);
     count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t level_residual(const MGLevel& L, double sigma, int nc, const double* w, const double* r, int64_t ldr,
-                           double* tmp, double* out, cudaStream_t s) {
-    const Grid& g = L.g;
-    int64_t total = g.n() * nc;
-    G3 G = g3(g);
-    bool d3 = g.d == 3;
-    if (!L.poly) {
-        if (L.shifted) {
-            if (d3) k_resid_lap<true, true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, w, r, ldr, out, total);
-            else k_resid_lap<false, true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, w, r, ldr, out, total);
-        } else {
-            if (d3) k_resid_lap<true, false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), 0.0, w, r, ldr, out, total);
-            else k_resid_lap<false, false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), 0.0, w, r, ldr, out, total);
-        }
-        count_launches(1);
-        return cudaGetLastError();
-    }
-    if (d3) k_shifted<true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, w, tmp, total);
-    else k_shifted<false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, w, tmp, total);
-    count_launches(1);
-    if (d3) k_poly_step<true><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, L.c, L.omega, 1, w, tmp, r, ldr, out, total);
-    else k_poly_step<false><<<nblk(total), kT, 0, s>>>(G, nc, g.inv_h2(), sigma, L.c, L.omega, 1, w, tmp, r, ldr, out, total);
-    count_launches(1);
-    return cudaGetLastError();
+// CTAs of the line transfers: up to 32 columns, segments whose fine points fit
+// 32 KB (64 points of 32 columns, whole lines at the usual sizes)
+LineCut line_cut(const Grid& gc, int nc) {
+    LineCut k;
+    k.cols = nc < 32 ? nc : 32;
+    const int64_t fit = 32 * 1024 / (int64_t)sizeof(double) / k.cols / 2 - 1;
+    k.seg = (int)(fit < gc.nx ? fit : gc.nx);
+    return k;
+}
+dim3 line_grid(int64_t lines, const Grid& gc, int nc, const LineCut& k) {
+    return dim3((unsigned)lines, (unsigned)((nc + k.cols - 1) / k.cols), (unsigned)((gc.nx + k.seg - 1) / k.seg));
 }
 
 // largest coarsest grid whose two work vectors are staged in shared memory
@@ -386,6 +390,8 @@ constexpr int64_t kCoarseShmPoints = kMaxSmemCoarse;
 cudaError_t coarse_solve(const MGHierarchy& H, int nc, const double* in, int64_t ldi, double* out, int64_t ldo,
                          double* gwork, cudaStream_t s) {
     const Grid& g = H.lev[0].g;
+    if (ldo == nc && coarse_split<CoarseF64>(g, nc))
+        return coarse_solve_split<CoarseF64>(g, nc, H.d_basis, H.d_mu, H.sigma, H.indefinite, in, ldi, out, s);
     int64_t n0 = g.n();
     const bool global = n0 > kCoarseShmPoints;
     size_t shm = global ? 0 : sizeof(double) * 2 * n0;
@@ -410,35 +416,47 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const double* r, int64_t
     const MGLevel& Lc = H.lev[l - 1];
     LevelBufs& b = B[l];
     cudaError_t e;
-    // pre-smoothing from zero
+    const Grid& g = L.g;
+    const double ih2 = g.inv_h2(), om = L.omega;
+    // pre-smoothing from zero; on a level without the polynomial the first two
+    // sweeps are one: 2 om r - om^2 B r
     double* cur = b.w0;
     double* nxt = b.w1;
-    e = rich_sweep(L, H.sigma, nc, nullptr, r, ldr, b.tmp, cur, s);
-    if (e != cudaSuccess) return e;
-    for (int i = 1; i < H.nu; ++i) {
-        e = rich_sweep(L, H.sigma, nc, cur, r, ldr, b.tmp, nxt, s);
+    int done = 1;
+    if (!L.poly && H.nu >= 2) {
+        const double diag = 2.0 * g.d * ih2 - (L.shifted ? H.sigma : 0.0);
+        launch_stencil(g, nc, 2.0 * om - om * om * diag, om * om * ih2, 0.0, r, ldr, nullptr, 0, cur, s);
+        done = 2;
+    } else {
+        k_scale<<<nblk(g.n() * nc), kT, 0, s>>>(nc, om, r, ldr, cur, g.n() * nc);
+        count_launches(1);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int i = done; i < H.nu; ++i) {
+        e = level_step(L, H.sigma, nc, 1.0, om, cur, r, ldr, b.tmp, nxt, s);
         if (e != cudaSuccess) return e;
         double* t = cur; cur = nxt; nxt = t;
     }
     // coarse-grid correction
-    e = level_residual(L, H.sigma, nc, cur, r, ldr, b.tmp, nxt, s);
+    e = level_step(L, H.sigma, nc, 0.0, 1.0, cur, r, ldr, b.tmp, nxt, s);
     if (e != cudaSuccess) return e;
-    int64_t totc = Lc.g.n() * nc;
-    if (L.g.d == 3) k_restrict<true><<<nblk(totc), kT, 0, s>>>(g3(L.g), g3(Lc.g), nc, H.linear, nxt, b.rc, totc);
-    else k_restrict<false><<<nblk(totc), kT, 0, s>>>(g3(L.g), g3(Lc.g), nc, H.linear, nxt, b.rc, totc);
+    const LineCut cut = line_cut(Lc.g, nc);
+    const size_t sm = sizeof(double) * 2 * (cut.seg + 1) * cut.cols;
+    const dim3 gr = line_grid(Lc.g.ny * Lc.g.nz, Lc.g, nc, cut), gp = line_grid(g.ny * g.nz, Lc.g, nc, cut);
+    if (g.d == 3) k_restrict_line<true><<<gr, kT, sm, s>>>(g3(g), g3(Lc.g), nc, cut, H.linear, nxt, b.rc);
+    else k_restrict_line<false><<<gr, kT, sm, s>>>(g3(g), g3(Lc.g), nc, cut, H.linear, nxt, b.rc);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = vcycle(H, l - 1, nc, b.rc, nc, b.wc, B, s);
     if (e != cudaSuccess) return e;
-    int64_t tot = L.g.n() * nc;
-    if (L.g.d == 3) k_prolong_add<true><<<nblk(tot), kT, 0, s>>>(g3(L.g), g3(Lc.g), nc, H.linear, b.wc, cur, tot);
-    else k_prolong_add<false><<<nblk(tot), kT, 0, s>>>(g3(L.g), g3(Lc.g), nc, H.linear, b.wc, cur, tot);
+    if (g.d == 3) k_prolong_line<true><<<gp, kT, sm, s>>>(g3(g), g3(Lc.g), nc, cut, H.linear, b.wc, cur);
+    else k_prolong_line<false><<<gp, kT, sm, s>>>(g3(g), g3(Lc.g), nc, cut, H.linear, b.wc, cur);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // post-smoothing; the last step writes to out
     for (int i = 0; i < H.nu; ++i) {
         double* dst = (i == H.nu - 1) ? out : nxt;
-        e = rich_sweep(L, H.sigma, nc, cur, r, ldr, b.tmp, dst, s);
+        e = level_step(L, H.sigma, nc, 1.0, om, cur, r, ldr, b.tmp, dst, s);
         if (e != cudaSuccess) return e;
         nxt = cur;
         cur = dst;

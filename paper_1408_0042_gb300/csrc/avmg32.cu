@@ -11,6 +11,7 @@
 // 64-bit index division is needed.  The two pre-smoothing sweeps from w = 0 on
 // an L_l level are fused: w = 2 omega r - omega^2 L r.
 #include "dword.h"
+#include "mgcoarse.h"
 #include "plhr_internal.h"
 
 namespace plhr {
@@ -504,6 +505,8 @@ struct Bufs {
 template <typename Tr>
 cudaError_t coarse(const MGHierarchy& H, int nc, const Tr* r, int64_t ldr, float* out, cudaStream_t s) {
     const Grid& g = H.lev[0].g;
+    if (coarse_split<CoarseF32>(g, nc))
+        return coarse_solve_split<CoarseF32>(g, nc, H.f_basis, H.f_mu, (float)H.sigma, 0, r, ldr, out, s);
     const size_t shm = sizeof(float) * 2 * g.n();
     if (shm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_coarse_sep<Tr>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);

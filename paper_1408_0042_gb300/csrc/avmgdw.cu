@@ -8,6 +8,7 @@
 // faster than FP64 arithmetic, which is bound by GB300's FP64 pipe.
 // The FP64 right-hand side is converted once; the result is converted back.
 #include "dword.h"
+#include "mgcoarse.h"
 #include "plhr_internal.h"
 
 namespace plhr {
@@ -18,6 +19,17 @@ constexpr int kT = 256;
 struct Ld {
     int nx, ny, nz, nc;
     dw ih2;
+};
+
+struct CoarseDw {
+    using V = dw;
+    static __device__ __forceinline__ V zero() { return dw_make(0.0f); }
+    static __device__ __forceinline__ void madd(V& s, V a, V b) { s = dw_add(s, dw_mul(a, b)); }
+    static __device__ __forceinline__ V scale(V x, V mx, V my, V mz, V sig, int) {
+        V den = dw_sub(dw_add(dw_add(mx, my), mz), sig);
+        if (den.hi < 0.0f) den = dw_neg(den);
+        return dw_div(x, den);
+    }
 };
 
 struct Pos {
@@ -428,6 +440,13 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, co
                    cudaStream_t s) {
     if (l == 0) {
         const Grid& g0 = H.lev[0].g;
+        if (coarse_split<CoarseDw>(g0, nc)) {
+            const dw* S[3] = {reinterpret_cast<const dw*>(H.w_basis[0]), reinterpret_cast<const dw*>(H.w_basis[1]),
+                              reinterpret_cast<const dw*>(H.w_basis[2])};
+            const dw* m[3] = {reinterpret_cast<const dw*>(H.w_mu[0]), reinterpret_cast<const dw*>(H.w_mu[1]),
+                              reinterpret_cast<const dw*>(H.w_mu[2])};
+            return coarse_solve_split<CoarseDw>(g0, nc, S, m, dw_host(H.sigma), 0, r, (int64_t)nc, out, s);
+        }
         const size_t shm = sizeof(dw) * 2 * g0.n();
         if (shm > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_coarse_sep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
