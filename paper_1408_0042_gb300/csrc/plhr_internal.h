@@ -221,10 +221,13 @@ struct SpecPrec {
     int d = 3;
     int64_t nx = 1, ny = 1, nz = 1;
     double energy = 1.0;
-    // double-word (hi, lo) FP32 pairs
-    float* d_S[3] = {nullptr, nullptr, nullptr};     // N_a x N_a, [point][mode]
-    float* d_St[3] = {nullptr, nullptr, nullptr};    // transposes
-    float* d_K = nullptr;                            // factor K(mu / energy) per 3D mode (n pairs)
+    bool periodic = false;
+    // double-word (hi, lo) FP32 pairs: the class matrices of each axis's plan,
+    // [folded point][mode] and [mode][folded point], and the factor
+    // K(mu / energy) per 3D mode in the plans' mode order
+    float* d_S[3] = {nullptr, nullptr, nullptr};
+    float* d_St[3] = {nullptr, nullptr, nullptr};
+    float* d_K = nullptr;
     int64_t n() const { return nx * ny * nz; }
 };
 cudaError_t spectral_apply(const SpecPrec& P, int nc, const double* r, int64_t ldr, double* w, double* work,
