@@ -17,6 +17,7 @@
 // INV-MG (Appendix A, Algorithm 5; H.indefinite): the same cycle with
 // B_l = L_l - sigma I_l on every level (the shift enters the sweeps and the
 // residual) and the signed coarsest solve S diag(1 / (mu - sigma)) S^T.
+#include "fxsum.h"
 #include "mgcoarse.h"
 #include "plhr_internal.h"
 
@@ -90,6 +91,32 @@ __global__ void __launch_bounds__(kT) k_stencil(G3 g, int nc, double cx, double 
         if (R) v = fma(cr, r[row * ldr + c], v);
         out[row * nc + c] = fma(cx, xp[0], v);
     }
+}
+
+// The two for blocks on which the FP64 pipe binds: the neighbours are summed on the
+// integer pipes, which leaves five FP64 operations of eight in a sweep (64^3 x 16: a
+// sweep 69 -> 51 us, the first two 61 -> 41, FP64 pipe 71-75 % and integer ALU 45-59 %
+// busy).
+template <bool D3, bool R>
+__global__ void __launch_bounds__(kFxThreads) k_stencil_fx(FxBox g, int nc, int planes, double cx, double cn, double cr,
+                                                           const double* __restrict__ x, int64_t ldx,
+                                                           const double* __restrict__ r, int64_t ldr,
+                                                           double* __restrict__ out) {
+    fx_walk<D3, false>(g, nc, planes, cn, x, ldx, [&](int64_t row, int c, double xc, double v) {
+        if (R) v = fma(cr, r[row * ldr + c], v);
+        out[row * nc + c] = fma(cx, xc, v);
+    });
+}
+template <bool D3>
+__global__ void __launch_bounds__(kFxThreads) k_poly_fx(FxBox g, int nc, int planes, double cw, double cr, double ct,
+                                                        double cn, const double* __restrict__ w,
+                                                        const double* __restrict__ t, const double* __restrict__ r,
+                                                        int64_t ldr, double* __restrict__ out) {
+    fx_walk<D3, false>(g, nc, planes, cn, t, nc, [&](int64_t row, int c, double tc, double v) {
+        v = fma(ct, tc, v);
+        v = fma(cw, w[row * nc + c], v);
+        out[row * nc + c] = fma(cr, r[row * ldr + c], v);
+    });
 }
 
 // w = om r (one sweep from zero)
@@ -338,7 +365,14 @@ void launch_stencil(const Grid& g, int nc, double cx, double cn, double cr, cons
     const int64_t total = g.n() * nc;
     const G3 G = g3(g);
     const int nb = nblk(total);
-    if (g.d == 3) {
+    const FxBox box{g.nx, g.ny, g.nz, 0};
+    if (const int planes = fx_planes(g.d, box, nc, cn)) {
+        auto go = [&](auto kern) {
+            kern<<<fx_grid(g.d, box, nc, planes), kFxThreads, 0, s>>>(box, nc, planes, cx, cn, cr, x, ldx, r, ldr, out);
+        };
+        if (g.d == 3) go(r ? k_stencil_fx<true, true> : k_stencil_fx<true, false>);
+        else go(r ? k_stencil_fx<false, true> : k_stencil_fx<false, false>);
+    } else if (g.d == 3) {
         if (r) k_stencil<true, true><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
         else k_stencil<true, false><<<nb, kT, 0, s>>>(G, nc, cx, cn, cr, x, ldx, r, ldr, out, total);
     } else {
@@ -361,7 +395,12 @@ cudaError_t level_step(const MGLevel& L, double sigma, int nc, double cw, double
     launch_stencil(g, nc, diag - sigma, -ih2, 0.0, w, nc, nullptr, 0, tmp, s);
     const double cb = cr / (2.0 * L.c);   // weight of (L - sig) t + c^2 w
     const int64_t total = g.n() * nc;
-    if (g.d == 3)
+    const FxBox box{g.nx, g.ny, g.nz, 0};
+    if (const int planes = fx_planes(g.d, box, nc, cb * ih2)) {
+        auto kern = g.d == 3 ? k_poly_fx<true> : k_poly_fx<false>;
+        kern<<<fx_grid(g.d, box, nc, planes), kFxThreads, 0, s>>>(box, nc, planes, cw - cb * L.c * L.c, cr,
+                                                                  -cb * (diag - sigma), cb * ih2, w, tmp, r, ldr, out);
+    } else if (g.d == 3)
         k_poly_step<true><<<nblk(total), kT, 0, s>>>(g3(g), nc, cw - cb * L.c * L.c, cr, -cb * (diag - sigma), cb * ih2,
                                                      w, tmp, r, ldr, out, total);
     else

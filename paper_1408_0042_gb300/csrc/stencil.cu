@@ -6,9 +6,10 @@
 // z), so a warp covers 32 consecutive doubles of the block, every neighbour
 // access of a warp (x +- 1: +-ld, y +- 1: +-ld*nx, z +- 1: +-ld*nx*ny) is one
 // contiguous 256-byte segment, the plane/line reuse is served from L1/L2, and
-// no 64-bit index division is needed.  The kernels are bound by GB300's FP64
-// pipe, so the FP64 operations per element are kept to seven: five additions
-// of the neighbours, one fused 2d x_c - sum, one scaling by 1/h^2.
+// no 64-bit index division is needed.  Seven FP64 operations an element: five
+// additions of the neighbours, one fused 2d x_c - sum, one scaling by 1/h^2.
+// On large blocks they would bind, and the sum runs on the integer pipes.
+#include "fxsum.h"
 #include "plhr_internal.h"
 
 namespace plhr {
@@ -106,6 +107,45 @@ __global__ void __launch_bounds__(256) k_lap_shifts(Geo g, int nc, double ih2, c
     if (o2) o2[e.row * ld2 + e.c] = fma(-sig, xv, a);
 }
 
+// The same products for blocks on which the FP64 pipe binds, summed on the integer
+// pipes (128^3 x 16: 515 -> 227 us, FP64 pipe 72 % and integer ALU 79 % busy).  MODE 0: y = alpha (L + pot) x + beta x,
+// mode as above; MODE 1: the shifted products.
+template <bool D3, int MODE, bool POT>
+__global__ void __launch_bounds__(kFxThreads) k_lap_fx(FxBox g, const double* __restrict__ pot, int nc, int planes,
+                                                       double ih2, const double* __restrict__ x, int64_t ldx,
+                                                       double* __restrict__ y, int64_t ldy, double alpha, double beta,
+                                                       int mode, double* __restrict__ o1, int64_t ld1,
+                                                       const double* __restrict__ lam, double* __restrict__ o2,
+                                                       int64_t ld2, double sig) {
+    fx_walk<D3, true>(g, nc, planes, ih2, x, ldx, [&](int64_t row, int c, double xc, double a) {
+        if (POT) a = fma(pot[row], xc, a);
+        if (MODE == 0) {
+            if (mode == 1) a *= alpha;
+            else if (mode == 2) a = fma(alpha, a, beta * xc);
+            y[row * ldy + c] = a;
+        } else {
+            if (y) y[row * ldy + c] = a;
+            if (o1) o1[row * ld1 + c] = fma(-lam[c], xc, a);
+            if (o2) o2[row * ld2 + c] = fma(-sig, xc, a);
+        }
+    });
+}
+
+FxBox box_of(const Grid& g) { return {g.nx, g.ny, g.nz, g.periodic}; }
+
+template <int MODE>
+void fx_launch(const Grid& g, int nc, int planes, const double* x, int64_t ldx, double* y, int64_t ldy, double alpha,
+               double beta, int mode, double* o1, int64_t ld1, const double* lam, double* o2, int64_t ld2, double sig,
+               cudaStream_t s) {
+    const FxBox b = box_of(g);
+    auto go = [&](auto kern) {
+        kern<<<fx_grid(g.d, b, nc, planes), kFxThreads, 0, s>>>(b, g.pot, nc, planes, g.inv_h2(), x, ldx, y, ldy, alpha,
+                                                                beta, mode, o1, ld1, lam, o2, ld2, sig);
+    };
+    if (g.d == 3) go(g.pot ? k_lap_fx<true, MODE, true> : k_lap_fx<true, MODE, false>);
+    else go(g.pot ? k_lap_fx<false, MODE, true> : k_lap_fx<false, MODE, false>);
+}
+
 dim3 grid_of(const Grid& g, int nc) {
     return dim3((unsigned)((g.nx * nc + 255) / 256), (unsigned)g.ny, (unsigned)g.nz);
 }
@@ -133,7 +173,9 @@ cudaError_t lap_axpby(const Grid& g, int nc, const double* x, int64_t ldx, doubl
     if (!grid_fits(g, nc)) return cudaErrorInvalidValue;
     Geo G = geo_of(g);
     const int mode = beta != 0.0 ? 2 : (alpha != 1.0 ? 1 : 0);
-    if (g.d == 3)
+    if (const int planes = fx_planes(g.d, box_of(g), nc, g.inv_h2()))
+        fx_launch<0>(g, nc, planes, x, ldx, y, ldy, alpha, beta, mode, nullptr, 0, nullptr, nullptr, 0, 0.0, s);
+    else if (g.d == 3)
         k_lap_axpby<true><<<grid_of(g, nc), 256, 0, s>>>(G, nc, g.inv_h2(), x, ldx, y, ldy, alpha, beta, mode);
     else
         k_lap_axpby<false><<<grid_of(g, nc), 256, 0, s>>>(G, nc, g.inv_h2(), x, ldx, y, ldy, alpha, beta, mode);
@@ -149,7 +191,9 @@ cudaError_t lap_apply_shifts(const Grid& g, int nc, const double* x, int64_t ldx
     if (g.n() * nc == 0) return cudaSuccess;
     if (!grid_fits(g, nc)) return cudaErrorInvalidValue;
     Geo G = geo_of(g);
-    if (g.d == 3)
+    if (const int planes = fx_planes(g.d, box_of(g), nc, g.inv_h2()))
+        fx_launch<1>(g, nc, planes, x, ldx, ax, ldax, 1.0, 0.0, 0, o1, ld1, lam, o2, ld2, sig, s);
+    else if (g.d == 3)
         k_lap_shifts<true><<<grid_of(g, nc), 256, 0, s>>>(G, nc, g.inv_h2(), x, ldx, ax, ldax, o1, ld1, lam, o2,
                                                            ld2, sig);
     else
