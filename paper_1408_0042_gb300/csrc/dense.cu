@@ -265,37 +265,75 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
 }
 
 // ---------------------------------------------------------------- eigenvalues (one warp)
-// Householder vector for (x, y[, z]) in double-word arithmetic: u = (1, u1, u2)
-// and tau with (I - tau u u^T)(x, y, z)^T = (beta, 0, 0)^T.
-__device__ __forceinline__ void house3(dw x, dw y, dw z, int nr, dw& u1, dw& u2, dw& tau) {
+// Householder vector for (x, y, z) in double-word arithmetic: u = (1, u1, u2),
+// tau and beta with (I - tau u u^T)(x, y, z)^T = (beta, 0, 0)^T.
+//
+// This is the longest part of a bulge step's dependent chain (double-word sums
+// are ten FP32 operations deep), so it is written with as few of them as the
+// accuracy allows: the squares are summed unnormalised, the square root and
+// the two reciprocals take one correction from FP32 and one from the
+// double-word remainder (their leading parts are correctly rounded after the
+// first, so the differences in the second are exact), and the reciprocal of
+// |x| + ||.|| starts from the FP32 norm, beside the norm's own corrections.
+// Relative errors stay below 2^-44 as with the general operations.
+__device__ __forceinline__ dw recip_refine(dw w, float r) {   // 1 / w, r its FP32 approximation
+    const float e = __fmaf_rn(-w.lo, r, __fmaf_rn(-w.hi, r, 1.0f));
+    dw q = dw_fast_two_sum(r, __fmul_rn(e, r));
+    const float p = __fmul_rn(w.hi, q.hi), pe = __fmaf_rn(w.hi, q.hi, -p);
+    const float t = __fmaf_rn(-w.lo, q.hi, __fmaf_rn(-w.hi, q.lo, -pe));
+    return dw_fast_two_sum(q.hi, __fmaf_rn(__fadd_rn(__fsub_rn(1.0f, p), t), r, q.lo));
+}
+__device__ __forceinline__ void house3(dw x, dw y, dw z, dw& u1, dw& u2, dw& tau, dw& beta) {
     const dw zero = dw_make(0.0f);
-    if (dw_is_zero(y) && (nr == 2 || dw_is_zero(z))) {
-        u1 = zero; u2 = zero; tau = zero;
+    if (dw_is_zero(y) && dw_is_zero(z)) {
+        u1 = zero; u2 = zero; tau = zero; beta = x;
         return;
     }
     // u and tau do not depend on the scale of (x, y, z): bring the largest to
     // about 1 by a power of two (exact) so that the squares stay inside FP32's
     // exponent range
+    const float mx = fmaxf(fabsf(x.hi), fmaxf(fabsf(y.hi), fabsf(z.hi)));
+    const float sc = pow2_inverse_of(mx);
+    const float sg = x.hi > 0.0f ? 1.0f : -1.0f;
+    x = dw_mul_pow2(x, __fmul_rn(sc, sg));   // |x|
+    y = dw_mul_pow2(y, sc);
+    z = dw_mul_pow2(z, sc);
+    const dw px = dw_two_prod(x.hi, x.hi), py = dw_two_prod(y.hi, y.hi), pz = dw_two_prod(z.hi, z.hi);
+    const float lx = __fmaf_rn(2.0f * x.hi, x.lo, px.lo), ly = __fmaf_rn(2.0f * y.hi, y.lo, py.lo),
+                lz = __fmaf_rn(2.0f * z.hi, z.lo, pz.lo);
+    const dw s1 = dw_two_sum(px.hi, py.hi), s2 = dw_two_sum(s1.hi, pz.hi);
+    const dw ss = dw_fast_two_sum(s2.hi, __fadd_rn(__fadd_rn(lx, ly), __fadd_rn(__fadd_rn(s1.lo, lz), s2.lo)));
+    // norm
+    const float rs = rsqrtf(ss.hi), hr = 0.5f * rs;
+    const float f = __fmul_rn(ss.hi, rs);
+    const float rw = __fdividef(1.0f, __fadd_rn(x.hi, f));
+    dw nrm = dw_fast_two_sum(f, __fmul_rn(__fadd_rn(__fmaf_rn(-f, f, ss.hi), ss.lo), hr));
     {
-        const float mx = fmaxf(fabsf(x.hi), fmaxf(fabsf(y.hi), nr == 3 ? fabsf(z.hi) : 0.0f));
-        const float sc = pow2_inverse_of(mx);
-        x = dw_mul_pow2(x, sc);
-        y = dw_mul_pow2(y, sc);
-        z = dw_mul_pow2(z, sc);
+        const float p = __fmul_rn(nrm.hi, nrm.hi), pe = __fmaf_rn(nrm.hi, nrm.hi, -p);
+        const float t = __fsub_rn(__fmaf_rn(-2.0f * nrm.hi, nrm.lo, ss.lo), pe);
+        nrm = dw_fast_two_sum(nrm.hi, __fmaf_rn(__fadd_rn(__fsub_rn(ss.hi, p), t), hr, nrm.lo));
     }
-    dw ss = dw_add(dw_mul(x, x), dw_mul(y, y));
-    if (nr == 3) ss = dw_add(ss, dw_mul(z, z));
-    dw nrm = dw_sqrt(ss);
-    if (dw_is_zero(nrm)) {
-        u1 = zero; u2 = zero; tau = zero;
-        return;
-    }
-    dw beta = x.hi > 0.0f ? dw_neg(nrm) : nrm;
-    dw v0 = dw_sub(x, beta);
-    dw rv = dw_div(dw_make(1.0f), v0);
-    u1 = dw_mul(y, rv);
-    u2 = nr == 3 ? dw_mul(z, rv) : zero;
-    tau = dw_div(dw_neg(v0), beta);   // (beta - x) / beta
+    // w = |x| + norm; u = sg (y, z) / w, tau = w / norm, beta = -sg norm
+    const dw h = dw_fast_two_sum(nrm.hi, x.hi);
+    const dw w = dw_fast_two_sum(h.hi, __fadd_rn(__fadd_rn(nrm.lo, x.lo), h.lo));
+    const dw rv = recip_refine(w, rw);
+    const dw rn = recip_refine(nrm, rs);
+    const dw srv = dw_mul_pow2(rv, sg);
+    u1 = dw_mul(y, srv);
+    u2 = dw_mul(z, srv);
+    tau = dw_mul(w, rn);
+    beta = dw_mul_pow2(nrm, -sg / sc);
+}
+
+// (a0 + u1 a1 + u2 a2) tau: the products' leading parts by error-free sums, everything
+// below them in FP32, normalised once
+__device__ __forceinline__ dw house_dot(dw a0, dw a1, dw a2, dw u1, dw u2, dw tau) {
+    const dw p = dw_two_prod(u1.hi, a1.hi), q = dw_two_prod(u2.hi, a2.hi);
+    const float lp = __fmaf_rn(u1.hi, a1.lo, __fmaf_rn(u1.lo, a1.hi, p.lo));
+    const float lq = __fmaf_rn(u2.hi, a2.lo, __fmaf_rn(u2.lo, a2.hi, q.lo));
+    const dw s = dw_two_sum(p.hi, q.hi), v = dw_two_sum(s.hi, a0.hi);
+    const float lo = __fadd_rn(__fadd_rn(__fadd_rn(lp, lq), __fadd_rn(s.lo, a0.lo)), v.lo);
+    return dw_mul(dw_two_sum(v.hi, lo), tau);
 }
 
 // Francis double-shift QR (Golub & Van Loan Sec. 7.5) on the upper Hessenberg
@@ -318,6 +356,7 @@ static_assert(kFrancisThreads >= MAXM, "one column / row per thread");
 
 __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* sweeps) {
     __shared__ double red[kFrancisThreads / 32];
+    __shared__ int last[kFrancisThreads / 32];
     const int t = threadIdx.x;
     double anorm = 0.0;
     for (int i = t; i < n * n; i += kFrancisThreads) {
@@ -349,14 +388,20 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
     int hi = n - 1;
     int its = 0, total_its = 0, total_steps = 0;
     while (hi >= 0) {
-        int l = hi;
-        while (l > 0) {
-            float s = fabsf(H[(l - 1) * LDS + l - 1].hi) + fabsf(H[l * LDS + l].hi);
-            if (s < hnorm) s = hnorm;
-            if (fabsf(H[l * LDS + l - 1].hi) <= eps * s) break;
-            --l;
+        // l = the last row at or above hi whose subdiagonal entry is negligible
+        // (row 0 always is), found by all threads at once
+        {
+            bool small = t == 0;
+            if (t > 0 && t <= hi) {
+                const float s = fmaxf(fabsf(H[(t - 1) * LDS + t - 1].hi) + fabsf(H[t * LDS + t].hi), hnorm);
+                small = fabsf(H[t * LDS + t - 1].hi) <= eps * s;
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, small);
+            if ((t & 31) == 0) last[t >> 5] = b ? (t & ~31) + 31 - __clz(b) : 0;
         }
         __syncthreads();
+        int l = 0;
+        for (int w = 0; w < kFrancisThreads / 32; ++w) l = max(l, last[w]);
         if (l > 0 && t == 0) H[l * LDS + l - 1] = zero;
         __syncthreads();
         if (l >= hi - 1) {          // 1x1 or 2x2 block converged
@@ -407,42 +452,42 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
         // any thread writes
         __syncthreads();
         for (int k = l; k <= hi - 1; ++k) {
-            const int nr = (k < hi - 1) ? 3 : 2;
-            dw u1, u2, tau;
-            house3(x, y, z, nr, u1, u2, tau);
-            if (!dw_is_zero(tau)) {
-                // left: rows k..k+2, column c0 + t
-                const int c0 = k > l ? k - 1 : l;
-                {
-                    const int ca = c0 + t;
-                    if (ca <= hi) {
-                        const dw a0 = H[k * LDS + ca], a1 = H[(k + 1) * LDS + ca];
-                        const dw a2 = nr == 3 ? H[(k + 2) * LDS + ca] : zero;
-                        const dw sa = dw_mul(dw_add(dw_add(a0, dw_mul(u1, a1)), dw_mul(u2, a2)), tau);
-                        H[k * LDS + ca] = dw_sub(a0, sa);
-                        H[(k + 1) * LDS + ca] = dw_sub(a1, dw_mul(sa, u1));
-                        if (nr == 3) H[(k + 2) * LDS + ca] = dw_sub(a2, dw_mul(sa, u2));
-                    }
-                }
-                __syncthreads();
-                // right: columns k..k+2, row l + t (rows l..min(k+3, hi))
-                const int r1 = (k + 3 < hi) ? k + 3 : hi;
-                {
-                    const int ra = l + t;
-                    if (ra <= r1) {
-                        const dw a0 = H[ra * LDS + k], a1 = H[ra * LDS + k + 1];
-                        const dw a2 = nr == 3 ? H[ra * LDS + k + 2] : zero;
-                        const dw sa = dw_mul(dw_add(dw_add(a0, dw_mul(u1, a1)), dw_mul(u2, a2)), tau);
-                        H[ra * LDS + k] = dw_sub(a0, sa);
-                        H[ra * LDS + k + 1] = dw_sub(a1, dw_mul(sa, u1));
-                        if (nr == 3) H[ra * LDS + k + 2] = dw_sub(a2, dw_mul(sa, u2));
-                    }
-                }
-                __syncthreads();
+            // rows (columns) k..k+2, the last step's k and k+1 with u2 = 0
+            const bool three = k < hi - 1;
+            // this thread's column of the left reflection (k..hi) is read before the
+            // reflector is formed
+            const int ca = k + t;
+            const bool left = ca <= hi;
+            dw a0 = zero, a1 = zero, a2 = zero;
+            if (left) {
+                a0 = H[k * LDS + ca];
+                a1 = H[(k + 1) * LDS + ca];
+                if (three) a2 = H[(k + 2) * LDS + ca];
             }
-            if (k > l && t == 0) {
+            dw u1, u2, tau, beta;
+            house3(x, y, three ? z : zero, u1, u2, tau, beta);
+            if (left) {
+                const dw sa = house_dot(a0, a1, a2, u1, u2, tau);
+                H[k * LDS + ca] = dw_sub(a0, sa);
+                H[(k + 1) * LDS + ca] = dw_sub(a1, dw_mul(sa, u1));
+                if (three) H[(k + 2) * LDS + ca] = dw_sub(a2, dw_mul(sa, u2));
+            }
+            __syncthreads();
+            // column k - 1 becomes (beta, 0, 0); every thread has read it above
+            if (k > l && t == kFrancisThreads - 1) {
+                H[k * LDS + k - 1] = beta;
                 H[(k + 1) * LDS + k - 1] = zero;
-                if (nr == 3) H[(k + 2) * LDS + k - 1] = zero;
+                if (three) H[(k + 2) * LDS + k - 1] = zero;
+            }
+            // right: row l + t (rows l..min(k+3, hi))
+            const int ra = l + t;
+            if (ra <= (k + 3 < hi ? k + 3 : hi)) {
+                dw* h = H + ra * LDS + k;
+                const dw b0 = h[0], b1 = h[1], b2 = three ? h[2] : zero;
+                const dw sb = house_dot(b0, b1, b2, u1, u2, tau);
+                h[0] = dw_sub(b0, sb);
+                h[1] = dw_sub(b1, dw_mul(sb, u1));
+                if (three) h[2] = dw_sub(b2, dw_mul(sb, u2));
             }
             __syncthreads();
             if (k < hi - 1) {
@@ -450,7 +495,6 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
                 y = H[(k + 2) * LDS + k];
                 z = (k < hi - 2) ? H[(k + 3) * LDS + k] : zero;
             }
-            __syncthreads();
         }
     }
     __syncthreads();
