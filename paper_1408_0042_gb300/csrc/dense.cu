@@ -322,7 +322,7 @@ __device__ __forceinline__ void house3(dw x, dw y, dw z, dw& u1, dw& u2, dw& tau
     u1 = dw_mul(y, srv);
     u2 = dw_mul(z, srv);
     tau = dw_mul(w, rn);
-    beta = dw_mul_pow2(nrm, -sg / sc);
+    beta = dw_mul_pow2(nrm, __fmul_rn(-sg, pow2_inverse_of(sc)));   // sc is a power of two
 }
 
 // (a0 + u1 a1 + u2 a2) tau: the products' leading parts by error-free sums, everything
@@ -646,7 +646,7 @@ struct Smem {
 // words of the shared-memory state saved to global memory between the launches
 constexpr int kStateWords = (int)(sizeof(Smem) / sizeof(int));
 static_assert(sizeof(Smem) % sizeof(int) == 0, "state copy granularity");
-// Yre, Yim, Yp (MAXM^2 each), then the saved state; a selected unit (at most
+// Yre, Yim (MAXM^2 each; MAXM^2 unused), then the saved state; a selected unit (at most
 // MAXKP) keeps its packed complex LU factor (MAXM (MAXM+1) / 2) in shared memory
 constexpr int MAXKP = 16;
 constexpr size_t kLuComplex = (size_t)MAXM * (MAXM + 1) / 2;
@@ -704,29 +704,21 @@ __device__ void dense_csolve_dw(double* Xd, const double* L, double* Lwd, double
     (void)lane;
 }
 
-// The dense stage runs as five launches: phase 0 of k_extract (up to the
-// Hessenberg form, state saved to global scratch), k_francis (two warps: the
-// eigenvalues), phase 1 (selection, state saved), k_eigvec (one CTA per
-// selected unit, in parallel), phase 2 (orthogonalisation, Y', coefficients).
-// The eigenvalue iteration measured 2x slower per bulge step when run inside
-// the large kernel than as its own launch on the same data and code, and the
-// eigenvectors ran four rounds on four warps of one SM.
-__global__ void __launch_bounds__(NT) k_extract(DenseArgs a, int phase) {
+// The dense stage runs as four launches: k_extract (up to the Hessenberg form,
+// state saved to global scratch), k_francis (two warps: the eigenvalues and the
+// selection), k_eigvec and k_finish (one CTA per selected unit each: the
+// eigenvector; cluster orthogonalisation, Y' and the coefficients of the unit's
+// columns).  The eigenvalue iteration measured 2x slower per bulge step when run
+// inside the large kernel than as its own launch on the same data and code.
+__global__ void __launch_bounds__(NT) k_extract(DenseArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& S = *reinterpret_cast<Smem*>(smem_raw);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     const int m = a.m, kp = a.kp;
     int* gst = reinterpret_cast<int*>(state_of(a));
     int* sst = reinterpret_cast<int*>(&S);
     int nk = 0, nvk = 0;
-    // global scratch: complex eigenvector coefficients per selected unit and Y'
-    double* Yre = a.work;                          // [unit][MAXM]
-    double* Yim = Yre + MAXM * MAXM;               // [unit][MAXM]
-    double* Yp = Yim + MAXM * MAXM;                // [col][MAXM]
-    double* Wr = Yre;                              // reused after Y' is assembled
-    double* Wv = Yim;
 #define STAMP(i) do { if (a.clk && tid == 0) a.clk[i] = clock64(); } while (0)
-  if (phase == 0) {
     STAMP(0);
     // ---- 1. B-orthonormalisation of Z, implicitly: Cholesky with column
     // dropping of the column-normalised Gram (the Grams are of Z diag(colscale)).
@@ -820,248 +812,6 @@ __global__ void __launch_bounds__(NT) k_extract(DenseArgs a, int phase) {
     if (tid == 0) S.ints[6] = 0;
     bsync();
     for (int i = tid; i < kStateWords; i += NT) gst[i] = sst[i];
-    return;
-  }
-    // ---- phases 1, 2: reload the state (the eigenvalues are in S.H, S.ints[2])
-    for (int i = tid; i < kStateWords; i += NT) sst[i] = gst[i];
-    bsync();
-    if (S.ints[6]) return;            // an earlier phase stopped (status already written)
-    nk = S.ints[0];
-    nvk = S.ints[1];
-  if (phase == 1) {
-    if (!S.ints[2]) {
-        if (tid == 0) { a.out_int[0] = kDenseNoConv; a.out_int[1] = nk; a.out_int[2] = 0; state_of(a)->ints[6] = 1; }
-        return;
-    }
-    // ---- 4. order by |xi| (xi = 1/tau), conjugate pairs adjacent, select k'
-    if (tid == 0) {
-        int q = 0, i = 0;
-        while (i < nk) {
-            if (i + 1 < nk && S.H[(i + 1) * LDS + i] != 0.0) {
-                double aa = S.H[i * LDS + i], bb = S.H[i * LDS + i + 1], cc = S.H[(i + 1) * LDS + i],
-                       dd = S.H[(i + 1) * LDS + i + 1];
-                double hf = 0.5 * (aa - dd), disc = hf * hf + bb * cc;
-                if (disc >= 0.0) {   // deflated block with two real eigenvalues
-                    double sq = sqrt(disc);
-                    S.eig_re[q] = 0.5 * (aa + dd) + sq; S.eig_im[q] = 0.0; ++q;
-                    S.eig_re[q] = 0.5 * (aa + dd) - sq; S.eig_im[q] = 0.0; ++q;
-                } else {
-                    // tau = re -+ i im: the member with Im(tau) < 0 has Im(xi) > 0
-                    S.eig_re[q] = 0.5 * (aa + dd); S.eig_im[q] = -sqrt(-disc); ++q;
-                    S.eig_re[q] = 0.5 * (aa + dd); S.eig_im[q] = sqrt(-disc); ++q;
-                }
-                i += 2;
-            } else {
-                S.eig_re[q] = S.H[i * LDS + i]; S.eig_im[q] = 0.0; ++q;
-                i += 1;
-            }
-        }
-        // units: real eigenvalues and conjugate pairs (represented by Im(tau) < 0)
-        int nu = 0;
-        int unit_e[MAXM];
-        double key_abs[MAXM], key_re[MAXM];
-        for (int e = 0; e < nk; ++e) {
-            if (S.eig_im[e] > 0.0) continue;
-            double re = S.eig_re[e], im = S.eig_im[e], m2 = re * re + im * im;
-            double xr = m2 > 0.0 ? re / m2 : INFINITY, xim = m2 > 0.0 ? -im / m2 : 0.0;
-            key_abs[nu] = m2 > 0.0 ? hypot(xr, xim) : INFINITY;
-            key_re[nu] = xr;
-            unit_e[nu] = e;
-            ++nu;
-        }
-        for (int i2 = 1; i2 < nu; ++i2) {
-            double ka = key_abs[i2], kr = key_re[i2];
-            int ue = unit_e[i2];
-            int j = i2 - 1;
-            while (j >= 0 && (key_abs[j] > ka || (key_abs[j] == ka && key_re[j] > kr))) {
-                key_abs[j + 1] = key_abs[j]; key_re[j + 1] = key_re[j]; unit_e[j + 1] = unit_e[j];
-                --j;
-            }
-            key_abs[j + 1] = ka; key_re[j + 1] = kr; unit_e[j + 1] = ue;
-        }
-        int sel = 0, ns = 0;
-        for (int u = 0; u < nu && sel < kp; ++u) {
-            int e = unit_e[u];
-            bool pair = S.eig_im[e] != 0.0;
-            S.order[ns] = e;
-            S.kind[ns] = pair ? ((kp - sel >= 2) ? 2 : 1) : 0;
-            sel += pair ? 2 : 1;
-            ++ns;
-        }
-        // numerical clusters among the selected: later members get a shifted
-        // inverse iteration and are orthogonalised against earlier ones
-        for (int u = 0; u < ns; ++u) {
-            int c = 0;
-            double re = S.eig_re[S.order[u]], im = S.eig_im[S.order[u]];
-            double mag = fmax(fabs(re) + fabs(im), 1e-300);
-            for (int v = 0; v < u; ++v) {
-                double d = fabs(S.eig_re[S.order[v]] - re) + fabs(S.eig_im[S.order[v]] - im);
-                if (d <= 1e-8 * mag) ++c;
-            }
-            S.nclose[u] = c;
-        }
-        S.ints[3] = ns;
-        for (int u = 0; u < ns; ++u) {
-            int e = S.order[u];
-            double re = S.eig_re[e], im = S.eig_im[e], m2 = re * re + im * im;
-            a.xi[2 * u] = re / m2;
-            a.xi[2 * u + 1] = -im / m2;
-        }
-    }
-    bsync();
-    for (int i = tid; i < kStateWords; i += NT) gst[i] = sst[i];   // selection saved for k_eigvec
-    return;
-  }
-    const int nsel = S.ints[3];
-    STAMP(5);
-    // ---- 5. (k_eigvec) eigenvectors of the selected units are in Yre, Yim
-    bsync();
-    STAMP(6);
-    // ---- cluster orthogonalisation, pair rotation, unit norm (warp 0, in the
-    // orthonormal basis: plain complex inner products)
-    if (warp == 0) {
-        for (int u = 0; u < nsel; ++u) {
-            double* yr = Yre + u * MAXM;
-            double* yi = Yim + u * MAXM;
-            // two passes of modified Gram-Schmidt against the earlier members
-            // of the cluster (the second restores the orthogonality the first
-            // loses when most of y lies in their span)
-            for (int pass = 0; pass < 2 && S.nclose[u] > 0; ++pass) {
-                const int e = S.order[u];
-                const double re = S.eig_re[e], im = S.eig_im[e];
-                const double mag = fmax(fabs(re) + fabs(im), 1e-300);
-                for (int v = 0; v < u; ++v) {
-                    const int f = S.order[v];
-                    if (fabs(S.eig_re[f] - re) + fabs(S.eig_im[f] - im) > 1e-8 * mag) continue;
-                    const double* vr = Yre + v * MAXM;
-                    const double* vi = Yim + v * MAXM;
-                    // y -= v (v^H y) / (v^H v)
-                    double pr = 0.0, pi = 0.0, vv = 0.0;
-                    for (int i = lane; i < nk; i += 32) {
-                        pr += vr[i] * yr[i] + vi[i] * yi[i];
-                        pi += vr[i] * yi[i] - vi[i] * yr[i];
-                        vv += vr[i] * vr[i] + vi[i] * vi[i];
-                    }
-                    pr = warp_sum(pr); pi = warp_sum(pi); vv = warp_sum(vv);
-                    pr /= vv; pi /= vv;
-                    for (int i = lane; i < nk; i += 32) {
-                        double ar = vr[i] * pr - vi[i] * pi, ai = vr[i] * pi + vi[i] * pr;
-                        yr[i] -= ar;
-                        yi[i] -= ai;
-                    }
-                    __threadfence_block();
-                    wsync();
-                }
-            }
-            double aa = 0.0, bb = 0.0, ab = 0.0;
-            for (int i = lane; i < nk; i += 32) { aa += yr[i] * yr[i]; bb += yi[i] * yi[i]; ab += yr[i] * yi[i]; }
-            aa = warp_sum(aa); bb = warp_sum(bb); ab = warp_sum(ab);
-            double c = 1.0, sn = 0.0;
-            if (S.kind[u] != 0) {
-                double phi = 0.5 * atan2(-2.0 * ab, aa - bb);
-                c = cos(phi); sn = sin(phi);
-            }
-            double nrm = sqrt(aa + bb);
-            if (!(nrm > 0.0)) nrm = 1.0;
-            for (int i = lane; i < nk; i += 32) {
-                double r = yr[i], im2 = yi[i];
-                yr[i] = (r * c - im2 * sn) / nrm;
-                yi[i] = (r * sn + im2 * c) / nrm;
-            }
-            __threadfence_block();
-            wsync();
-        }
-    }
-    bsync();
-    // ---- Y' = [Y0 YR yR~ YI] (kept basis), column tags: thread 0 assigns the
-    // columns of each unit (keep: real part, nclose: imaginary part or -1;
-    // both free after the cluster step), then every thread copies entries
-    if (tid == 0) {
-        int nreal = 0, npair = 0;
-        bool has_cut = false;
-        for (int u = 0; u < nsel; ++u) {
-            if (S.kind[u] == 0) ++nreal;
-            else if (S.kind[u] == 2) ++npair;
-            else has_cut = true;
-        }
-        int col = 0, pr = 0;
-        const int base_R = nreal, base_cut = nreal + npair, base_I = nreal + npair + (has_cut ? 1 : 0);
-        for (int u = 0; u < nsel; ++u) {
-            if (S.kind[u] == 0) {
-                S.keep[u] = col; S.nclose[u] = -1;
-                a.tags[col] = 0; a.tag_partner[col] = -1;
-                ++col;
-            } else if (S.kind[u] == 2) {
-                const int cr = base_R + pr, ci = base_I + pr;
-                S.keep[u] = cr; S.nclose[u] = ci;
-                a.tags[cr] = 1; a.tag_partner[cr] = ci;
-                a.tags[ci] = 3; a.tag_partner[ci] = cr;
-                ++pr;
-            } else {
-                S.keep[u] = base_cut; S.nclose[u] = -1;
-                a.tags[base_cut] = 2; a.tag_partner[base_cut] = -1;
-            }
-        }
-    }
-    bsync();
-    for (int idx = tid; idx < nsel * nk; idx += NT) {
-        const int u = idx / nk, i = idx - u * nk;
-        Yp[S.keep[u] * MAXM + i] = Yre[u * MAXM + i];
-        if (S.nclose[u] >= 0) Yp[S.nclose[u] * MAXM + i] = Yim[u * MAXM + i];
-    }
-    __threadfence_block();
-    bsync();
-    STAMP(7);
-    // ---- 6. raw coefficients.  Z-hat = Z diag(colscale t) R^{-1}; R^{-1} is
-    // upper triangular with the V columns first, so
-    //   P_new = Z-hat[:, rest] Y'_rest = Z diag(colscale t) R^{-1} [0; Y'_rest]
-    //   V_new - P_new = Z-hat[:, V] Y'_V = Z_V diag(colscale t) R_VV^{-1} Y'_V
-    // Four lanes per solve split each inner sum (l mod 4) and combine it by two
-    // shuffles: column j = 4 warp + (g & 3) of lane group g = lane / 4, groups
-    // 0..3 solve for Wr and 4..7 for Wv, all in one instruction stream (an
-    // FP64 warp instruction costs the same whatever its active lanes, so a
-    // quarter of the terms per lane is a quarter of the time); the diagonal's
-    // reciprocals are formed once, in parallel.
-    static_assert(MAXKP <= 16, "four warps of four columns");
-    for (int i = tid; i < nk; i += NT) S.red[i] = 1.0 / S.A[i * LDS + i];
-    bsync();
-    {
-        const int g4 = lane & 3, grp = lane >> 2;
-        const int j = warp * 4 + (grp & 3);
-        const bool isv = grp >= 4;
-        double* W = isv ? Wv : Wr;
-        const int lim = isv ? nvk : nk;
-        for (int i = nk - 1; i >= 0; --i) {
-            const bool act = j < kp && i < lim;
-            double part = 0.0;
-            if (act)
-                for (int l = i + 1 + g4; l < lim; l += 4) part = fma(-S.A[i * LDS + l], W[j * MAXM + l], part);
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            if (act && g4 == 0) {
-                const double y = (isv || i >= nvk) ? Yp[j * MAXM + i] : 0.0;
-                W[j * MAXM + i] = (y + part) * S.red[i];
-            }
-            __syncwarp();
-        }
-    }
-    for (int i = tid; i < m * kp; i += NT) a.Cp[i] = 0.0;
-    for (int i = tid; i < a.nv * kp; i += NT) a.Cvv[i] = 0.0;
-    __threadfence_block();
-    bsync();
-    for (int i = tid; i < nk * kp; i += NT) {
-        const int q = i / kp, j = i % kp;
-        const int raw = S.kidx[q];
-        const double tr = S.t[raw] * a.colscale[raw];
-        a.Cp[raw * kp + j] = tr * Wr[j * MAXM + q];
-        if (q < nvk) a.Cvv[raw * kp + j] = tr * Wv[j * MAXM + q];
-    }
-    STAMP(8);
-    if (tid == 0) {
-        a.out_int[0] = kDenseOK;
-        a.out_int[1] = nk;
-        a.out_int[2] = nsel;
-    }
 #undef STAMP
 }
 
@@ -1164,29 +914,260 @@ __global__ void __launch_bounds__(32) k_eigvec(DenseArgs a) {
     }
 }
 
-// Eigenvalues of the saved Hessenberg form (two warps; see k_extract).  The
-// stage clocks 3 and 4 and the sweep counts come from this launch.
+// Order by |xi| (xi = 1/tau), conjugate pairs adjacent, select k': the eigenvalues
+// are in the diagonal blocks of H (n x n).  Every step takes one thread per
+// eigenvalue, unit or rank (one thread for all of it took 180 us).
+static_assert(kFrancisThreads >= MAXM, "one eigenvalue per thread");
+__device__ void select_units(const DenseArgs& a, Smem* G, const double* H, int n) {
+    __shared__ double er[MAXM], ei[MAXM], ka[MAXM], kr[MAXM];
+    __shared__ int slot[MAXM], size[MAXM], order[MAXM], count;
+    const int t = threadIdx.x, kp = a.kp;
+    if (t == 0) count = 0;
+    if (t < MAXM) { slot[t] = 0; size[t] = 0; }
+    __syncthreads();
+    const bool own = t < n;
+    double re = 0.0, im = 0.0;
+    if (own) {
+        const bool second = t > 0 && H[t * LDS + t - 1] != 0.0;
+        const bool first = !second && t + 1 < n && H[(t + 1) * LDS + t] != 0.0;
+        if (first || second) {
+            const double* b = H + (t - (second ? 1 : 0)) * (LDS + 1);
+            const double aa = b[0], bb = b[1], cc = b[LDS], dd = b[LDS + 1];
+            const double hf = 0.5 * (aa - dd), disc = hf * hf + bb * cc, mean = 0.5 * (aa + dd);
+            const double sq = sqrt(fabs(disc));
+            // two real eigenvalues, or tau = re -+ i im: the member with
+            // Im(tau) < 0, which has Im(xi) > 0, first
+            re = disc >= 0.0 ? (second ? mean - sq : mean + sq) : mean;
+            im = disc >= 0.0 ? 0.0 : (second ? sq : -sq);
+        } else {
+            re = H[t * LDS + t];
+        }
+        er[t] = re; ei[t] = im;
+        G->eig_re[t] = re; G->eig_im[t] = im;
+    }
+    // units: real eigenvalues and conjugate pairs (represented by Im(tau) < 0)
+    const bool unit = own && !(im > 0.0);
+    const double m2 = re * re + im * im;
+    if (own) {
+        const double xr = m2 > 0.0 ? re / m2 : INFINITY, xim = m2 > 0.0 ? -im / m2 : 0.0;
+        ka[t] = m2 > 0.0 ? hypot(xr, xim) : INFINITY;
+        kr[t] = xr;
+    }
+    __syncthreads();
+    if (unit) {
+        const double k = ka[t], x = kr[t];
+        int rank = 0;
+        for (int v = 0; v < n; ++v)
+            rank += !(ei[v] > 0.0) && (ka[v] < k || (ka[v] == k && (kr[v] < x || (kr[v] == x && v < t))));
+        slot[rank] = t;
+        size[rank] = im != 0.0 ? 2 : 1;
+    }
+    __syncthreads();
+    int sel = 0;
+    if (own) {
+        for (int q = 0; q < t; ++q) sel += size[q];
+        if (size[t] > 0 && sel < kp) {
+            order[t] = slot[t];
+            G->order[t] = slot[t];
+            G->kind[t] = size[t] == 2 ? (kp - sel >= 2 ? 2 : 1) : 0;
+            atomicAdd(&count, 1);
+        }
+    }
+    __syncthreads();
+    const int ns = count;   // the ranks below ns are selected
+    if (t < ns) {
+        const int e = order[t];
+        const double tre = er[e], tim = ei[e], t2 = tre * tre + tim * tim;
+        // numerical clusters among the selected: later members get a shifted
+        // inverse iteration and are orthogonalised against earlier ones
+        const double mag = fmax(fabs(tre) + fabs(tim), 1e-300);
+        int c = 0;
+        for (int v = 0; v < t; ++v) c += fabs(er[order[v]] - tre) + fabs(ei[order[v]] - tim) <= 1e-8 * mag;
+        G->nclose[t] = c;
+        a.xi[2 * t] = tre / t2;
+        a.xi[2 * t + 1] = -tim / t2;
+    }
+    if (t == 0) G->ints[3] = ns;
+}
+
+// Eigenvalues of the saved Hessenberg form (two warps; see k_extract) and the
+// selection.  The stage clocks 3 and 4 and the sweep counts come from this launch.
 __global__ void __launch_bounds__(kFrancisThreads) k_francis(DenseArgs a) {
     extern __shared__ __align__(16) double shh[];
     Smem* G = state_of(a);
     if (G->ints[6]) return;
     const int nk = G->ints[0];
     const int t = threadIdx.x;
-    for (int i = t; i < nk * LDS; i += kFrancisThreads) shh[i] = G->H[i];
+    for (int i = t; i < nk * LDS; i += kFrancisThreads) shh[i] = G->H0[i];
     __syncthreads();
     if (a.clk && t == 0) a.clk[3] = clock64();
     const bool conv = francis_eigenvalues(shh, nk, a.clk ? a.clk + 9 : nullptr);
     if (a.clk && t == 0) a.clk[4] = clock64();
-    for (int i = t; i < nk * LDS; i += kFrancisThreads) G->H[i] = shh[i];
-    if (t == 0) G->ints[2] = conv ? 1 : 0;
+    if (conv) {
+        select_units(a, G, shh, nk);
+    } else if (t == 0) {
+        a.out_int[0] = kDenseNoConv; a.out_int[1] = nk; a.out_int[2] = 0; G->ints[6] = 1;
+    }
+}
+
+// Two selected units belong to one numerical cluster (u the later one)
+__device__ __forceinline__ bool close_units(const Smem* G, int u, int v) {
+    const int e = G->order[u], f = G->order[v];
+    const double mag = fmax(fabs(G->eig_re[e]) + fabs(G->eig_im[e]), 1e-300);
+    return fabs(G->eig_re[f] - G->eig_re[e]) + fabs(G->eig_im[f] - G->eig_im[e]) <= 1e-8 * mag;
+}
+
+// Cluster orthogonalisation, pair rotation, unit norm of unit u and the
+// coefficients of its one or two columns of Y' = [Y0 YR yR~ YI] (CTA u).  A
+// member of a cluster needs the earlier members' final vectors: its CTA works
+// them out again from the raw ones (clusters are small, and one warp doing the
+// units in turn took 75 us).  The back substitutions (real and imaginary column,
+// for P_new and V_new - P_new, a warp each) subtract a solved entry from all rows
+// at once: two FP64 operations deep a row instead of a sum (59 us; the whole
+// stage, with the state's copy, 185 -> 25 us at m = 64, 16 columns).
+__global__ void __launch_bounds__(128) k_finish(DenseArgs a) {
+    extern __shared__ __align__(16) double shy[];
+    double* R = shy;                  // MAXM x LDS
+    double* Y = R + MAXM * LDS;       // [unit][re, im][MAXM]
+    __shared__ double rinv[MAXM], W[4][MAXM];
+    const Smem* G = state_of(a);
+    if (G->ints[6]) return;
+    const int nk = G->ints[0], nvk = G->ints[1], nsel = G->ints[3];
+    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (u >= nsel) return;
+    if (a.clk && u == 0 && tid == 0) { a.clk[5] = clock64(); a.clk[6] = a.clk[5]; }
+    for (int i = tid; i < nk * LDS; i += 128) R[i] = G->A[i];
+    const double* Yre = a.work;
+    const double* Yim = a.work + MAXM * MAXM;
+    if (warp == 0) {
+        unsigned need = 1u << u;
+        for (int v = u; v > 0; --v)
+            if ((need >> v & 1u) && G->nclose[v] > 0)
+                for (int w = 0; w < v; ++w)
+                    if (close_units(G, v, w)) need |= 1u << w;
+        for (int v = 0; v <= u; ++v) {
+            if (!(need >> v & 1u)) continue;
+            double* yr = Y + v * 2 * MAXM;
+            double* yi = yr + MAXM;
+            for (int i = lane; i < nk; i += 32) { yr[i] = Yre[v * MAXM + i]; yi[i] = Yim[v * MAXM + i]; }
+            wsync();
+            // two passes of modified Gram-Schmidt against the earlier members
+            // of the cluster (the second restores the orthogonality the first
+            // loses when most of y lies in their span); plain complex inner
+            // products, in the orthonormal basis
+            for (int pass = 0; pass < 2 && G->nclose[v] > 0; ++pass)
+                for (int w = 0; w < v; ++w) {
+                    if (!close_units(G, v, w)) continue;
+                    const double* vr = Y + w * 2 * MAXM;
+                    const double* vi = vr + MAXM;
+                    // y -= v (v^H y) / (v^H v)
+                    double pr = 0.0, pi = 0.0, vv = 0.0;
+                    for (int i = lane; i < nk; i += 32) {
+                        pr += vr[i] * yr[i] + vi[i] * yi[i];
+                        pi += vr[i] * yi[i] - vi[i] * yr[i];
+                        vv += vr[i] * vr[i] + vi[i] * vi[i];
+                    }
+                    pr = warp_sum(pr); pi = warp_sum(pi); vv = warp_sum(vv);
+                    pr /= vv; pi /= vv;
+                    for (int i = lane; i < nk; i += 32) {
+                        const double ar = vr[i] * pr - vi[i] * pi, ai = vr[i] * pi + vi[i] * pr;
+                        yr[i] -= ar;
+                        yi[i] -= ai;
+                    }
+                    wsync();
+                }
+            double aa = 0.0, bb = 0.0, ab = 0.0;
+            for (int i = lane; i < nk; i += 32) { aa += yr[i] * yr[i]; bb += yi[i] * yi[i]; ab += yr[i] * yi[i]; }
+            aa = warp_sum(aa); bb = warp_sum(bb); ab = warp_sum(ab);
+            double c = 1.0, sn = 0.0;
+            if (G->kind[v] != 0) {
+                const double phi = 0.5 * atan2(-2.0 * ab, aa - bb);
+                c = cos(phi); sn = sin(phi);
+            }
+            double nrm = sqrt(aa + bb);
+            if (!(nrm > 0.0)) nrm = 1.0;
+            for (int i = lane; i < nk; i += 32) {
+                const double re = yr[i], im = yi[i];
+                yr[i] = (re * c - im * sn) / nrm;
+                yi[i] = (re * sn + im * c) / nrm;
+            }
+            wsync();
+        }
+    } else {
+        for (int i = tid - 32; i < nk; i += 96) rinv[i] = 1.0 / G->A[i * LDS + i];
+    }
+    __syncthreads();
+    if (a.clk && u == 0 && tid == 0) a.clk[7] = clock64();
+    // columns of the unit: real part, imaginary part or -1
+    int nreal = 0, npair = 0, ncut = 0, before_real = 0, before_pair = 0;
+    for (int v = 0; v < nsel; ++v) {
+        const int k = G->kind[v];
+        if (v < u) { before_real += k == 0; before_pair += k == 2; }
+        nreal += k == 0; npair += k == 2; ncut += k == 1;
+    }
+    const int kind = G->kind[u];
+    const int cr = kind == 0 ? before_real : kind == 2 ? nreal + before_pair : nreal + npair;
+    const int ci = kind == 2 ? nreal + npair + ncut + before_pair : -1;
+    if (tid == 0) {
+        a.tags[cr] = kind == 0 ? 0 : kind == 2 ? 1 : 2;
+        a.tag_partner[cr] = ci;
+        if (ci >= 0) { a.tags[ci] = 3; a.tag_partner[ci] = cr; }
+    }
+    // ---- raw coefficients.  Z-hat = Z diag(colscale t) R^{-1}; R^{-1} is
+    // upper triangular with the V columns first, so
+    //   P_new = Z-hat[:, rest] Y'_rest = Z diag(colscale t) R^{-1} [0; Y'_rest]
+    //   V_new - P_new = Z-hat[:, V] Y'_V = Z_V diag(colscale t) R_VV^{-1} Y'_V
+    // warps 0, 1: P_new's real and imaginary column, 2, 3: V_new - P_new's
+    if ((warp & 1) == 0 || ci >= 0) {
+        const bool isv = warp >= 2;
+        const double* y = Y + (u * 2 + (warp & 1)) * MAXM;
+        const int lim = isv ? nvk : nk, r0 = lane, r1 = lane + 32;
+        double b0 = r0 < lim && (isv || r0 >= nvk) ? y[r0] : 0.0;
+        double b1 = r1 < lim && (isv || r1 >= nvk) ? y[r1] : 0.0;
+        for (int i = lim - 1; i >= 0; --i) {
+            const double w = __shfl_sync(0xffffffffu, i >= 32 ? b1 : b0, i & 31) * rinv[i];
+            if (r0 < i) b0 = fma(-R[r0 * LDS + i], w, b0);
+            if (i > 32) {
+                if (r1 < i) b1 = fma(-R[r1 * LDS + i], w, b1);
+            }
+            if (r0 == i) b0 = w;
+            if (r1 == i) b1 = w;
+        }
+        W[warp][r0] = b0;
+        W[warp][r1] = b1;
+    }
+    const int m = a.m, kp = a.kp;
+    for (int half = 0; half < 2; ++half) {
+        const int col = half ? ci : cr;
+        if (col < 0) break;
+        for (int i = tid; i < m; i += 128) a.Cp[i * kp + col] = 0.0;
+        for (int i = tid; i < a.nv; i += 128) a.Cvv[i * kp + col] = 0.0;
+    }
+    __syncthreads();
+    for (int half = 0; half < 2; ++half) {
+        const int col = half ? ci : cr;
+        if (col < 0) break;
+        for (int q = tid; q < nk; q += 128) {
+            const int raw = G->kidx[q];
+            const double tr = G->t[raw] * a.colscale[raw];
+            a.Cp[raw * kp + col] = tr * W[half][q];
+            if (q < nvk) a.Cvv[raw * kp + col] = tr * W[2 + half][q];
+        }
+    }
+    if (u == 0 && tid == 0) {
+        if (a.clk) a.clk[8] = clock64();
+        a.out_int[0] = kDenseOK;
+        a.out_int[1] = nk;
+        a.out_int[2] = nsel;
+    }
 }
 
 }  // namespace
 
 size_t dense_smem_bytes() { return sizeof(Smem); }
 
-// Yre, Yim, Yp (3 MAXM^2) and the shared-memory state passed between the
-// launches.
+// Yre, Yim (MAXM^2 each; MAXM^2 unused) and the shared-memory state passed
+// between the launches.
 size_t dense_work_doubles() { return kDenseWorkDoubles; }
 static_assert(kWorkMainDoubles >= 3 * (size_t)MAXM * MAXM, "dense scratch layout");
 
@@ -1200,12 +1181,14 @@ cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     const size_t she = sizeof(double) * kEigvecShmDoubles;
     e = cudaFuncSetAttribute(k_eigvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she);
     if (e != cudaSuccess) return e;
-    k_extract<<<1, NT, shm, s>>>(a, 0);
+    const size_t shn = sizeof(double) * (MAXM * LDS + MAXKP * 2 * MAXM);
+    e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shn);
+    if (e != cudaSuccess) return e;
+    k_extract<<<1, NT, shm, s>>>(a);
     k_francis<<<1, kFrancisThreads, shf, s>>>(a);
-    k_extract<<<1, NT, shm, s>>>(a, 1);
     k_eigvec<<<a.kp, 32, she, s>>>(a);
-    k_extract<<<1, NT, shm, s>>>(a, 2);
-    count_launches(5);
+    k_finish<<<a.kp, 128, shn, s>>>(a);
+    count_launches(4);
     return cudaGetLastError();
 }
 
