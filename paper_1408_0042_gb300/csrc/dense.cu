@@ -22,6 +22,8 @@
 #include "dense.h"
 #include "dword.h"
 
+#include <cooperative_groups.h>
+
 #include <cfloat>
 #include <mutex>
 
@@ -30,7 +32,7 @@ namespace {
 
 constexpr int MAXM = kDenseMaxM;
 constexpr int LDS = MAXM + 1;     // shared row stride: column accesses hit distinct banks
-constexpr int NT = 128;           // threads of the extraction CTA
+constexpr int NT = 512;           // threads of a k_pencil CTA
 
 __device__ __forceinline__ void wsync() { __syncwarp(); }
 __device__ __forceinline__ void bsync() { __syncthreads(); }
@@ -68,91 +70,93 @@ __device__ bool chol_lower(double* A, int n, int ld) {
 }
 
 // ---------------------------------------------------------------- block-wide dense kernels
-// Cholesky with column dropping of a symmetric n x n (upper triangle used):
-// A = R^T R on the kept columns; column j is dropped when its pivot is below
-// tol (the matrix is column-normalised, so the test is relative).
-__device__ int bchol_drop(double* A, int n, int* keep, double tol) {
+// r = sqrt(p) and ri = 1 / r, p > 0: an FP32 estimate and two Goldschmidt
+// iterations on p scaled by an even power of two, one Newton correction of the
+// root (P. Markstein, "Software division and square root using Goldschmidt's
+// algorithms", RNC 2004).  Eight dependent FP64 operations for both, where an FP64
+// warp instruction takes 64 cycles of its pipe.
+__device__ __forceinline__ void sqrt_and_inverse(double p, double& r, double& ri) {
+    const int hi = __double2hiint(p);
+    if (hi < 0x00100000) {   // subnormal
+        r = sqrt(p);
+        ri = 1.0 / r;
+        return;
+    }
+    const int e = ((hi >> 20) - 1023) & ~1;
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(p));   // in [1, 4)
+    const float y = rsqrtf((float)m);
+    double g = m * (double)y, h = (double)(0.5f * y);
+    for (int i = 0; i < 2; ++i) {
+        const double d = fma(-g, h, 0.5);
+        g = fma(g, d, g);
+        h = fma(h, d, h);
+    }
+    g = fma(fma(-g, g, m), h, g);
+    r = __hiloint2double(__double2hiint(g) + ((e / 2) << 20), __double2loint(g));
+    ri = __hiloint2double(__double2hiint(h) + ((1 - e / 2) << 20), __double2loint(h));
+}
+
+// Cholesky A = R^T R of a symmetric n x n (upper triangle used and replaced).
+// With keep, column j is dropped when its pivot is below tol (the matrix is
+// column-normalised, so the test is relative); without, a pivot that is not
+// above tol ends it (false).  Two warps on two sub-partitions form the pivot's
+// root and scale the row (one product and a correction with the remainder instead
+// of a division an entry), all warps update: the chain of a column is about 13
+// FP64 operations (64 columns: 291,000 -> 208,000 cycles).
+__device__ bool bchol(double* A, int n, int* keep, double tol) {
     const int tid = threadIdx.x;
-    int nk = 0;
     for (int j = 0; j < n; ++j) {
-        double p = A[j * LDS + j];
-        bool ok = (p > tol) && isfinite(p);
-        bsync();
-        if (tid == 0) keep[j] = ok ? 1 : 0;
-        if (ok) {
-            double r = sqrt(p);
-            for (int l = j + 1 + tid; l < n; l += NT) A[j * LDS + l] /= r;
+        const double p = A[j * LDS + j];
+        const bool ok = (p > tol) && isfinite(p);
+        if (!ok && !keep) {
             bsync();
-            if (tid == 0) A[j * LDS + j] = r;
-            const int w = n - j - 1;
-            for (int idx = tid; idx < w * w; idx += NT) {
-                int a = j + 1 + idx / w, b = j + 1 + idx % w;
-                if (b >= a) A[a * LDS + b] -= A[j * LDS + a] * A[j * LDS + b];
+            return false;
+        }
+        double r = 0.0;
+        if (ok && tid < 64) {
+            double ri;
+            sqrt_and_inverse(p, r, ri);
+            const int l = j + 1 + tid;
+            if (l < n) {
+                const double v = A[j * LDS + l], q = v * ri;
+                A[j * LDS + l] = fma(fma(-q, r, v), ri, q);
             }
-            ++nk;
+        }
+        bsync();
+        if (keep && tid == 0) keep[j] = ok ? 1 : 0;
+        if (ok) {
+            if (tid == 0) A[j * LDS + j] = r;
+            for (int a = j + 1 + (tid >> 4); a < n; a += NT / 16) {
+                const double f = A[j * LDS + a];
+                for (int b = a + (tid & 15); b < n; b += 16) A[a * LDS + b] = fma(-f, A[j * LDS + b], A[a * LDS + b]);
+            }
         } else {
             for (int l = tid; l < n; l += NT) A[j * LDS + l] = 0.0;
         }
         bsync();
     }
-    return nk;
-}
-
-// Column (row) index of this thread in the one-column-per-thread FP64 loops:
-// 16 lanes of each of the four warps, one warp per SM sub-partition, so that
-// all four FP64 pipes work (a warp instruction occupies the pipe for the same
-// time whatever its active lanes).  Lanes 16..31 take the same index of a
-// second matrix (spread_second).  Every index is handled by one thread, in
-// the same order as with one thread per index.
-static_assert(NT == 128 && MAXM <= 64, "four warps of 16 lanes cover the columns");
-__device__ __forceinline__ int spread_index() { return (threadIdx.x >> 5) * 16 + (threadIdx.x & 15); }
-__device__ __forceinline__ bool spread_second() { return (threadIdx.x & 16) != 0; }
-
-// X1 <- R^{-T} X1 R^{-1} and X2 <- R^{-T} X2 R^{-1} (X2 optional) for upper
-// triangular R (all n x n, stride LDS)
-__device__ void bcongruence2(const double* R, double* X1, double* X2, int n) {
-    const int c = spread_index();
-    double* X = spread_second() ? X2 : X1;
-    if (X != nullptr && c < n) {
-        for (int i = 0; i < n; ++i) {
-            double s = X[i * LDS + c];
-            for (int l = 0; l < i; ++l) s -= R[l * LDS + i] * X[l * LDS + c];
-            X[i * LDS + c] = s / R[i * LDS + i];
-        }
-    }
-    bsync();
-    if (X != nullptr && c < n) {
-        const int r = c;
-        for (int j = 0; j < n; ++j) {
-            double s = X[r * LDS + j];
-            for (int l = 0; l < j; ++l) s -= X[r * LDS + l] * R[l * LDS + j];
-            X[r * LDS + j] = s / R[j * LDS + j];
-        }
-    }
-    bsync();
-}
-
-// A = L L^T (lower triangle), block-wide; false when not positive definite
-__device__ bool bchol_lower(double* A, int n, int* flag) {
-    const int tid = threadIdx.x;
-    for (int j = 0; j < n; ++j) {
-        double p = A[j * LDS + j];
-        bool ok = (p > 0.0) && isfinite(p);
-        if (!ok) { bsync(); return false; }
-        double r = sqrt(p);
-        bsync();
-        for (int l = j + 1 + tid; l < n; l += NT) A[l * LDS + j] /= r;
-        bsync();
-        if (tid == 0) A[j * LDS + j] = r;
-        const int w = n - j - 1;
-        for (int idx = tid; idx < w * w; idx += NT) {
-            int a = j + 1 + idx / w, b = j + 1 + idx % w;
-            if (b <= a) A[a * LDS + b] -= A[a * LDS + j] * A[b * LDS + j];
-        }
-        bsync();
-    }
-    (void)flag;
     return true;
+}
+
+// Solves T x = b for a lower triangular T by one warp: b0, b1 are rows lane and
+// lane + 32 of b, then of x.  Tc[l * LDS + i] = T_il / T_ll (i > l), rinv_l = 1 / T_ll:
+// each unknown, unscaled, is subtracted from the rows below at once, one FP64
+// operation deep, and the scaling comes last.
+__device__ __forceinline__ void warp_solve(const double* Tc, const double* rinv, int n, double& b0, double& b1) {
+    const int lane = threadIdx.x & 31;
+    const int n0 = n < 32 ? n : 32;
+    for (int l = 0; l < n0; ++l) {
+        const double x = __shfl_sync(0xffffffffu, b0, l);
+        const double* t = Tc + l * LDS;
+        if (lane > l && lane < n) b0 = fma(-t[lane], x, b0);
+        if (lane + 32 < n) b1 = fma(-t[lane + 32], x, b1);
+    }
+    for (int l = 32; l < n; ++l) {
+        const double x = __shfl_sync(0xffffffffu, b1, l - 32);
+        if (lane + 32 > l && lane + 32 < n) b1 = fma(-Tc[l * LDS + lane + 32], x, b1);
+    }
+    if (lane < n) b0 *= rinv[lane];
+    if (lane + 32 < n) b1 *= rinv[lane + 32];
 }
 
 // Householder reduction of H (n x n) to upper Hessenberg form.  The reflector
@@ -164,10 +168,13 @@ __device__ bool bchol_lower(double* A, int n, int* flag) {
 // the double-word QR iteration that follows it, and the FP64 form (one
 // dependent FP64 chain per column, each warp instruction holding the FP64 pipe
 // for 64 cycles) cost about a million cycles at n = 64.  Every column and row
-// belongs to a pair of threads that split its sum over i by parity (lazily
-// normalised double-word sums, combined by one shuffle).  v and beta describe
-// the same reflector at any scale, so only H is scaled back; H, Vh and beta
-// are FP64 again on return.
+// belongs to eight threads that split its sum over i (lazily normalised
+// double-word sums, combined by three shuffles); columns c and c + 8 share a half
+// warp, so that its 16 accesses (odd stride) fall into distinct banks.  One warp
+// forms the reflector's scalars.  Four warps a scheduler hide each other's
+// dependent operations (two threads a column, one warp a scheduler: 522,000 ->
+// HESS_CYC cycles at n = 64).  v and beta describe the same reflector at any
+// scale, so only H is scaled back; H, Vh and beta are FP64 again on return.
 __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, double* red) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const dw zero = dw_make(0.0f);
@@ -189,9 +196,14 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
     }
     bsync();
     float* redf = reinterpret_cast<float*>(red);
-    const int own = tid >> 1, half = tid & 1;
+    const int part = lane & 7, own = (warp & 7) + 8 * (lane >> 3) + 32 * (warp >> 3);
+    auto sum8 = [](dw v) {
+        for (int o = 1; o < 8; o <<= 1)
+            v = dw_add(v, dw{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+        return v;
+    };
     for (int k = 0; k < n - 2; ++k) {
-        // ||x||^2 for x = H[k+1:n, k]  (warp 0)
+        // warp 0: ||x||^2 for x = H[k+1:n, k], beta and v_{k+1}
         if (warp == 0) {
             dwacc acc = {0.0f, 0.0f};
             for (int i = k + 1 + lane; i < n; i += 32) {
@@ -201,21 +213,26 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
             dw ss = dwacc_result(acc);
             for (int o = 16; o > 0; o >>= 1)
                 ss = dw_add(ss, dw{__shfl_xor_sync(0xffffffffu, ss.hi, o), __shfl_xor_sync(0xffffffffu, ss.lo, o)});
-            if (lane == 0) { redf[0] = ss.hi; redf[1] = ss.lo; }
+            const dw x0 = H[(k + 1) * LDS + k];
+            dw alpha = dw_sqrt(ss);
+            if (x0.hi > 0.0f) alpha = dw_neg(alpha);
+            // v_{k+1} = x0 - alpha, v^T v = 2 (ss - x0 alpha) (alpha^2 = ss, no
+            // cancellation: -x0 alpha >= 0), beta = 2 / v^T v
+            const dw den = dw_sub(ss, dw_mul(x0, alpha));
+            const bool none = dw_is_zero(alpha) || !(den.hi > 0.0f);
+            if (lane == 0) {
+                const dw b = none ? zero : dw_div(dw_make(1.0f), den), v0 = dw_sub(x0, alpha);
+                redf[0] = b.hi; redf[1] = b.lo;
+                redf[2] = v0.hi; redf[3] = v0.lo;
+                redf[4] = none ? 1.0f : 0.0f;
+                B[k] = b;
+            }
         }
         bsync();
-        const dw ss = {redf[0], redf[1]};
-        const dw x0 = H[(k + 1) * LDS + k];
-        dw alpha = dw_sqrt(ss);
-        if (x0.hi > 0.0f) alpha = dw_neg(alpha);
-        // v_{k+1} = x0 - alpha, v^T v = 2 (ss - x0 alpha) (alpha^2 = ss, no
-        // cancellation: -x0 alpha >= 0), beta = 2 / v^T v
-        const dw den = dw_sub(ss, dw_mul(x0, alpha));
-        const bool skip = dw_is_zero(alpha) || !(den.hi > 0.0f);
-        const dw b = skip ? zero : dw_div(dw_make(1.0f), den);
-        for (int i = tid; i < n; i += NT)
-            V[k * LDS + i] = (i <= k || skip) ? zero : (i == k + 1 ? dw_sub(x0, alpha) : H[i * LDS + k]);
-        if (tid == 0) B[k] = b;
+        const dw b = {redf[0], redf[1]};
+        const bool skip = redf[4] != 0.0f;
+        if (tid < n)
+            V[k * LDS + tid] = (tid <= k || skip) ? zero : (tid == k + 1 ? dw{redf[2], redf[3]} : H[tid * LDS + k]);
         bsync();
         if (!skip) {
             const dw* v = V + k * LDS;
@@ -225,12 +242,14 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
                 const bool act = c < n && c >= k;
                 dwacc acc = {0.0f, 0.0f};
                 if (act)
-                    for (int i = k + 1 + half; i < n; i += 2) dwacc_add_mul(acc, v[i], H[i * LDS + c]);
-                dw sv = dwacc_result(acc);
-                sv = dw_add(sv, dw{__shfl_xor_sync(0xffffffffu, sv.hi, 1), __shfl_xor_sync(0xffffffffu, sv.lo, 1)});
-                sv = dw_mul(sv, b);
+                    for (int i = k + 1 + part; i < n; i += 8) dwacc_add_mul(acc, v[i], H[i * LDS + c]);
+                const dw sv = dw_neg(dw_mul(sum8(dwacc_result(acc)), b));
                 if (act)
-                    for (int i = k + 1 + half; i < n; i += 2) H[i * LDS + c] = dw_sub(H[i * LDS + c], dw_mul(sv, v[i]));
+                    for (int i = k + 1 + part; i < n; i += 8) {
+                        dwacc h = dwacc_of(H[i * LDS + c]);
+                        dwacc_add_mul(h, sv, v[i]);
+                        H[i * LDS + c] = dwacc_result(h);
+                    }
             }
             bsync();
             // H <- H (I - b v v^T) : row r = own
@@ -239,14 +258,16 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
                 const bool act = r < n;
                 dwacc acc = {0.0f, 0.0f};
                 if (act)
-                    for (int i = k + 1 + half; i < n; i += 2) dwacc_add_mul(acc, H[r * LDS + i], v[i]);
-                dw sv = dwacc_result(acc);
-                sv = dw_add(sv, dw{__shfl_xor_sync(0xffffffffu, sv.hi, 1), __shfl_xor_sync(0xffffffffu, sv.lo, 1)});
-                sv = dw_mul(sv, b);
+                    for (int i = k + 1 + part; i < n; i += 8) dwacc_add_mul(acc, H[r * LDS + i], v[i]);
+                const dw sv = dw_neg(dw_mul(sum8(dwacc_result(acc)), b));
                 if (act)
-                    for (int i = k + 1 + half; i < n; i += 2) H[r * LDS + i] = dw_sub(H[r * LDS + i], dw_mul(sv, v[i]));
+                    for (int i = k + 1 + part; i < n; i += 8) {
+                        dwacc h = dwacc_of(H[r * LDS + i]);
+                        dwacc_add_mul(h, sv, v[i]);
+                        H[r * LDS + i] = dwacc_result(h);
+                    }
             }
-            bsync();
+            // column k below its subdiagonal entry is zero now; no row update reads it
             for (int i = k + 2 + tid; i < n; i += NT) H[i * LDS + k] = zero;
         }
         bsync();
@@ -624,194 +645,239 @@ __device__ __forceinline__ dw warp_sum_dw(dw v) {
     return v;
 }
 
-// ---------------------------------------------------------------- the kernel
-struct Smem {
-    double H[MAXM * LDS];     // C, then its Hessenberg form, then the quasi-triangular result
-    double H0[MAXM * LDS];    // Hessenberg form of C (kept for inverse iteration)
+// ---------------------------------------------------------------- the state between the launches
+struct DenseState {
+    double H[MAXM * LDS];     // G_R, then C
+    double H0[MAXM * LDS];    // Hessenberg form of C
     double Vh[MAXM * LDS];    // Householder vectors of the Hessenberg reduction
-    double A[MAXM * LDS];     // column-normalised B-Gram -> R
+    double A[MAXM * LDS];     // R (upper), the Cholesky factor of the kept columns' Gram
     double B[MAXM * LDS];     // G_L -> L
     double beta[MAXM];
     double t[MAXM];           // column normalisation of the (scaled) basis
-    double red[NT];
-    int keep[MAXM];
     int kidx[MAXM];           // kept -> raw index
     double eig_re[MAXM], eig_im[MAXM];
     int order[MAXM];          // selected units: eigenvalue index
     int kind[MAXM];           // 0 real, 2 full pair, 1 cut pair
     int nclose[MAXM];         // earlier selected units in the same numerical cluster
-    int ints[8];
+    int ints[8];              // [0] kept columns, [1] of V, [3] selected units, [6] stop, [7] pencil's verdict
 };
 
-// words of the shared-memory state saved to global memory between the launches
-constexpr int kStateWords = (int)(sizeof(Smem) / sizeof(int));
-static_assert(sizeof(Smem) % sizeof(int) == 0, "state copy granularity");
 // Yre, Yim (MAXM^2 each; MAXM^2 unused), then the saved state; a selected unit (at most
 // MAXKP) keeps its packed complex LU factor (MAXM (MAXM+1) / 2) in shared memory
 constexpr int MAXKP = 16;
 constexpr size_t kLuComplex = (size_t)MAXM * (MAXM + 1) / 2;
 constexpr size_t kWorkMainDoubles = 3 * (size_t)MAXM * MAXM;
-constexpr size_t kDenseWorkDoubles = kWorkMainDoubles + (sizeof(Smem) + sizeof(double) - 1) / sizeof(double);
+constexpr size_t kDenseWorkDoubles = kWorkMainDoubles + (sizeof(DenseState) + sizeof(double) - 1) / sizeof(double);
 
-__device__ __forceinline__ Smem* state_of(const DenseArgs& a) {
-    return reinterpret_cast<Smem*>(a.work + kWorkMainDoubles);
+__device__ __forceinline__ DenseState* state_of(const DenseArgs& a) {
+    return reinterpret_cast<DenseState*>(a.work + kWorkMainDoubles);
 }
 
-// X <- L^{-1} X L^{-T} for the n x n block X (stride LDS, FP64 in and out)
-// and the lower triangular L (FP64), in double-word arithmetic; Lw (n x LDS
-// double-word) and rinv (n double-word values) are scratch.  Block-wide.
-__device__ void dense_csolve_dw(double* Xd, const double* L, double* Lwd, double* rinvd, int n) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    dw* X = reinterpret_cast<dw*>(Xd);
-    dw* Lw = reinterpret_cast<dw*>(Lwd);
-    dw* rinv = reinterpret_cast<dw*>(rinvd);
-    for (int i = tid; i < n * n; i += NT) {
-        const int r = i / n, c = i % n;
-        X[r * LDS + c] = dw_from_double_fast(Xd[r * LDS + c]);
-        if (c <= r) Lw[r * LDS + c] = dw_from_double_fast(L[r * LDS + c]);
-    }
-    bsync();
-    for (int i = tid; i < n; i += NT) rinv[i] = dw_div(dw_make(1.0f), Lw[i * LDS + i]);
-    bsync();
-    const int own = tid >> 1, half = tid & 1;
-    const bool act = own < n;
-    // columns: X[i][c] = (X[i][c] - sum_{l<i} L[i][l] X[l][c]) / L[i][i]
-    for (int i = 0; i < n; ++i) {
-        dwacc acc = {0.0f, 0.0f};
-        if (act)
-            for (int l = half; l < i; l += 2) dwacc_add_mul(acc, Lw[i * LDS + l], X[l * LDS + own]);
-        dw sv = dwacc_result(acc);
-        sv = dw_add(sv, dw{__shfl_xor_sync(0xffffffffu, sv.hi, 1), __shfl_xor_sync(0xffffffffu, sv.lo, 1)});
-        if (act && half == 0) X[i * LDS + own] = dw_mul(dw_sub(X[i * LDS + own], sv), rinv[i]);
-        __syncwarp();
-    }
-    bsync();
-    // rows: X[r][j] = (X[r][j] - sum_{l<j} X[r][l] L[j][l]) / L[j][j]
-    for (int j = 0; j < n; ++j) {
-        dwacc acc = {0.0f, 0.0f};
-        if (act)
-            for (int l = half; l < j; l += 2) dwacc_add_mul(acc, X[own * LDS + l], Lw[j * LDS + l]);
-        dw sv = dwacc_result(acc);
-        sv = dw_add(sv, dw{__shfl_xor_sync(0xffffffffu, sv.hi, 1), __shfl_xor_sync(0xffffffffu, sv.lo, 1)});
-        if (act && half == 0) X[own * LDS + j] = dw_mul(dw_sub(X[own * LDS + j], sv), rinv[j]);
-        __syncwarp();
-    }
-    bsync();
-    for (int i = tid; i < n * n; i += NT) {
-        const int r = i / n, c = i % n;
-        Xd[r * LDS + c] = dw_to_double(X[r * LDS + c]);
-    }
-    (void)lane;
-}
-
-// The dense stage runs as four launches: k_extract (up to the Hessenberg form,
+// The dense stage runs as four launches: k_pencil (up to the Hessenberg form,
 // state saved to global scratch), k_francis (two warps: the eigenvalues and the
 // selection), k_eigvec and k_finish (one CTA per selected unit each: the
 // eigenvector; cluster orthogonalisation, Y' and the coefficients of the unit's
 // columns).  The eigenvalue iteration measured 2x slower per bulge step when run
 // inside the large kernel than as its own launch on the same data and code.
-__global__ void __launch_bounds__(NT) k_extract(DenseArgs a) {
+//
+// k_pencil is one cluster of kPencilCtas CTAs.  The first does the serial parts
+// (the two Cholesky factorisations, the Hessenberg form); the triangular solves,
+// one warp per column and then per row, are spread over all of them, since 512 solves
+// of 64 unknowns are half a million FP64 multiply-adds, 258,000 cycles of one SM's
+// FP64 pipe (both congruences 588,000 -> 109,000 cycles).  Blocks pass between the
+// CTAs through the global state; what another CTA wrote is read past L1.
+constexpr int kPencilCtas = 8;
+struct PencilShm {
+    double A[MAXM * LDS];    // column-normalised B-Gram, then G_L, and their factors
+    double T[MAXM * LDS];    // columns of a triangular factor over its diagonal
+    double H[MAXM * LDS];
+    double Vh[MAXM * LDS];
+    double beta[MAXM], t[MAXM], rinv[MAXM], red[NT / 32];
+    int keep[MAXM], kidx[MAXM];
+};
+
+// S.T, S.rinv from a factor in global memory: T_il at f[l * LDS + i] (upper, T = R^T)
+// or f[i * LDS + l] (lower)
+__device__ __forceinline__ void load_factor(PencilShm& S, const double* f, bool upper, int n) {
+    bsync();
+    for (int i = threadIdx.x; i < n; i += NT) S.rinv[i] = 1.0 / __ldcg(f + i * LDS + i);
+    bsync();
+    for (int e = threadIdx.x; e < n * n; e += NT) {
+        const int l = e / n, i = e - l * n;
+        if (i > l) S.T[l * LDS + i] = __ldcg(f + (upper ? l * LDS + i : i * LDS + l)) * S.rinv[l];
+    }
+    bsync();
+}
+
+__global__ void __cluster_dims__(kPencilCtas, 1, 1) __launch_bounds__(NT) k_pencil(DenseArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem& S = *reinterpret_cast<Smem*>(smem_raw);
-    const int tid = threadIdx.x;
+    PencilShm& S = *reinterpret_cast<PencilShm*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31;
     const int m = a.m, kp = a.kp;
-    int* gst = reinterpret_cast<int*>(state_of(a));
-    int* sst = reinterpret_cast<int*>(&S);
-    int nk = 0, nvk = 0;
-#define STAMP(i) do { if (a.clk && tid == 0) a.clk[i] = clock64(); } while (0)
+    const bool lead = blockIdx.x == 0;
+    const int solver = blockIdx.x * (NT / 32) + (tid >> 5);   // 2 MAXM warps of the cluster
+    static_assert(kPencilCtas * (NT / 32) == 2 * MAXM, "one warp per column of two blocks");
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    DenseState* G = state_of(a);
+    int nk = 0;
+#define STAMP(i) do { if (a.clk && lead && tid == 0) a.clk[i] = clock64(); } while (0)
     STAMP(0);
     // ---- 1. B-orthonormalisation of Z, implicitly: Cholesky with column
     // dropping of the column-normalised Gram (the Grams are of Z diag(colscale)).
     // The basis Z D R^{-1} amplifies Gram rounding by cond(R)^2; if G_L then is
     // not numerically positive definite the pass is repeated with a stricter
     // drop threshold.
-    for (int i = tid; i < m; i += NT) {
-        double g = a.Gzz[i * m + i];
-        S.t[i] = (g > 0.0 && isfinite(g)) ? 1.0 / sqrt(g) : 0.0;
+    if (lead) {
+        for (int i = tid; i < m; i += NT) {
+            const double g = a.Gzz[i * m + i];
+            S.t[i] = (g > 0.0 && isfinite(g)) ? 1.0 / sqrt(g) : 0.0;
+            G->t[i] = S.t[i];
+        }
     }
     bsync();
     const double drop_tols[3] = {1e-12, 1e-9, 1e-6};
-    bool ok = false;
-    for (int attempt = 0; attempt < 3 && !ok; ++attempt) {
-        for (int i = tid; i < m * m; i += NT) {
-            int r = i / m, c = i % m;
-            S.A[r * LDS + c] = a.Gzz[i] * S.t[r] * S.t[c];
-        }
-        bsync();
-        bchol_drop(S.A, m, S.keep, drop_tols[attempt]);
-        STAMP(11);
-        if (tid == 0) {
-            int q = 0, qv = 0;
-            for (int j = 0; j < m; ++j)
-                if (S.keep[j] && S.t[j] != 0.0) {
-                    S.kidx[q++] = j;
-                    if (j < a.nv) ++qv;
-                }
-            S.ints[0] = q;
-            S.ints[1] = qv;
-        }
-        bsync();
-        nk = S.ints[0];
-        nvk = S.ints[1];
-        if (nvk < 1 || nk < kp) break;
-        // compact R (upper) in place through H
-        for (int i = tid; i < nk * nk; i += NT) {
-            int r = i / nk, c = i % nk;
-            S.H[r * LDS + c] = (c >= r) ? S.A[S.kidx[r] * LDS + S.kidx[c]] : 0.0;
-        }
-        bsync();
-        for (int i = tid; i < nk * nk; i += NT) S.A[(i / nk) * LDS + i % nk] = S.H[(i / nk) * LDS + i % nk];
-        bsync();
-        // G_L = sym(U^T Q), G_R[r][c] = q_r . z_c, on the kept, normalised columns
-        for (int i = tid; i < nk * nk; i += NT) {
-            int r = i / nk, c = i % nk;
-            int rr = S.kidx[r], cc = S.kidx[c];
-            S.B[r * LDS + c] = 0.5 * (a.Guq[rr * m + cc] + a.Guq[cc * m + rr]) * S.t[rr] * S.t[cc];
-            S.H[r * LDS + c] = a.Gqz[rr * m + cc] * S.t[rr] * S.t[cc];
-        }
-        bsync();
-        // ---- 2. the pencil in the B-orthonormal basis, via tau = 1/xi
-        STAMP(12);
-        bcongruence2(S.A, S.B, S.H, nk);
-        STAMP(13);
-        for (int i = tid; i < nk * nk; i += NT) {
-            int r = i / nk, c = i % nk;
-            if (c > r) {
-                double sv = 0.5 * (S.B[r * LDS + c] + S.B[c * LDS + r]);
-                S.B[r * LDS + c] = sv;
-                S.B[c * LDS + r] = sv;
+    enum { PENCIL_OK = 0, PENCIL_AGAIN = 1, PENCIL_STOP = 2 };
+    int next = PENCIL_AGAIN;
+    for (int attempt = 0; attempt < 3 && next == PENCIL_AGAIN; ++attempt) {
+        if (lead) {
+            for (int i = tid; i < m * m; i += NT) {
+                const int r = i / m, c = i % m;
+                S.A[r * LDS + c] = a.Gzz[i] * S.t[r] * S.t[c];
+            }
+            bsync();
+            bchol(S.A, m, S.keep, drop_tols[attempt]);
+            STAMP(11);
+            if (tid == 0) {
+                int q = 0, qv = 0;
+                for (int j = 0; j < m; ++j)
+                    if (S.keep[j] && S.t[j] != 0.0) {
+                        S.kidx[q] = j;
+                        G->kidx[q++] = j;
+                        if (j < a.nv) ++qv;
+                    }
+                G->ints[0] = q;
+                G->ints[1] = qv;
+                const bool loss = qv < 1 || q < kp;
+                if (loss) { a.out_int[0] = kDenseRankLoss; a.out_int[1] = q; a.out_int[2] = 0; }
+                G->ints[6] = loss ? 1 : 0;
+                S.keep[0] = q;
+            }
+            bsync();
+            nk = S.keep[0];
+            // compact R (upper)
+            for (int i = tid; i < nk * nk; i += NT) {
+                const int r = i / nk, c = i % nk;
+                G->A[r * LDS + c] = (c >= r) ? S.A[S.kidx[r] * LDS + S.kidx[c]] : 0.0;
             }
         }
-        bsync();
-        ok = bchol_lower(S.B, nk, nullptr);
+        STAMP(12);
+        cluster.sync();
+        nk = __ldcg(&G->ints[0]);
+        if (__ldcg(&G->ints[6])) {
+            next = PENCIL_STOP;
+            break;
+        }
+        // ---- 2. the pencil in the B-orthonormal basis, via tau = 1/xi: G_L =
+        // sym(U^T Q), G_R[r][c] = q_r . z_c on the kept, normalised columns, by
+        // columns R^{-T} X, then by rows X R^{-1}
+        load_factor(S, G->A, true, nk);
+        {
+            const int c = solver & (MAXM - 1);
+            const bool gl = solver < MAXM;
+            double* X = gl ? G->B : G->H;
+            double b0 = 0.0, b1 = 0.0;
+            if (c < nk) {
+                const int cc = __ldcg(&G->kidx[c]);
+                const double tc = __ldcg(&G->t[cc]);
+                for (int half = 0; half < 2; ++half) {
+                    const int r = lane + 32 * half;
+                    if (r >= nk) break;
+                    const int rr = __ldcg(&G->kidx[r]);
+                    const double v = gl ? 0.5 * (a.Guq[rr * m + cc] + a.Guq[cc * m + rr]) : a.Gqz[rr * m + cc];
+                    (half ? b1 : b0) = v * __ldcg(&G->t[rr]) * tc;
+                }
+                warp_solve(S.T, S.rinv, nk, b0, b1);
+                if (lane < nk) X[lane * LDS + c] = b0;
+                if (lane + 32 < nk) X[(lane + 32) * LDS + c] = b1;
+            }
+            cluster.sync();
+            if (c < nk) {
+                double* x = X + c * LDS;
+                b0 = lane < nk ? __ldcg(x + lane) : 0.0;
+                b1 = lane + 32 < nk ? __ldcg(x + lane + 32) : 0.0;
+                warp_solve(S.T, S.rinv, nk, b0, b1);
+                if (lane < nk) x[lane] = b0;
+                if (lane + 32 < nk) x[lane + 32] = b1;
+            }
+        }
+        cluster.sync();
+        STAMP(13);
+        if (lead) {
+            for (int i = tid; i < nk * nk; i += NT) {
+                const int r = i / nk, c = i % nk;
+                if (c >= r) S.A[r * LDS + c] = 0.5 * (__ldcg(&G->B[r * LDS + c]) + __ldcg(&G->B[c * LDS + r]));
+            }
+            bsync();
+            const bool ok = bchol(S.A, nk, nullptr, 0.0);
+            if (ok) {
+                for (int i = tid; i < nk * nk; i += NT) {   // L = R^T
+                    const int r = i / nk, c = i % nk;
+                    G->B[r * LDS + c] = c <= r ? S.A[c * LDS + r] : 0.0;
+                }
+            }
+            if (tid == 0) G->ints[7] = ok ? PENCIL_OK : PENCIL_AGAIN;
+        }
+        cluster.sync();
+        next = __ldcg(&G->ints[7]);
     }
     STAMP(1);
-    if (nvk < 1 || nk < kp) {
-        if (tid == 0) { a.out_int[0] = kDenseRankLoss; a.out_int[1] = nk; a.out_int[2] = 0; state_of(a)->ints[6] = 1; }
+    if (next != PENCIL_OK) {
+        if (lead && tid == 0 && next == PENCIL_AGAIN) {
+            a.out_int[0] = kDenseBreakdown; a.out_int[1] = nk; a.out_int[2] = 0;
+            G->ints[6] = 1;
+        }
         return;
     }
-    if (!ok) {
-        if (tid == 0) { a.out_int[0] = kDenseBreakdown; a.out_int[1] = nk; a.out_int[2] = 0; state_of(a)->ints[6] = 1; }
-        return;
+    // C = L^{-1} G_R L^{-T}: by columns, then by rows, eight warps a CTA
+    load_factor(S, G->B, false, nk);
+    {
+        const int c = blockIdx.x * (MAXM / kPencilCtas) + (tid >> 5);
+        const bool act = (tid >> 5) < MAXM / kPencilCtas && c < nk;
+        double b0 = 0.0, b1 = 0.0;
+        if (act) {
+            if (lane < nk) b0 = __ldcg(&G->H[lane * LDS + c]);
+            if (lane + 32 < nk) b1 = __ldcg(&G->H[(lane + 32) * LDS + c]);
+            warp_solve(S.T, S.rinv, nk, b0, b1);
+            if (lane < nk) G->H[lane * LDS + c] = b0;
+            if (lane + 32 < nk) G->H[(lane + 32) * LDS + c] = b1;
+        }
+        cluster.sync();
+        if (act) {
+            double* x = G->H + c * LDS;
+            b0 = lane < nk ? __ldcg(x + lane) : 0.0;
+            b1 = lane + 32 < nk ? __ldcg(x + lane + 32) : 0.0;
+            warp_solve(S.T, S.rinv, nk, b0, b1);
+            if (lane < nk) x[lane] = b0;
+            if (lane + 32 < nk) x[lane + 32] = b1;
+        }
     }
-    // C = L^{-1} G_R L^{-T}: L Y = G_R by columns, then C L^T = Y by rows, in
-    // double-word arithmetic (L is the Cholesky factor of the SPD G_L in the
-    // B-orthonormal basis; its condition is the square root of G_L's, so the
-    // solves lose little; in FP64 each dependent chain held a warp's FP64 pipe
-    // for 64 cycles per step).  A pair of threads owns a column (then a row)
-    // and splits each inner sum by parity; L (double-word) goes into the
-    // H0 array, free until the Hessenberg form is copied there, the
-    // reciprocals of its diagonal into red.
-    dense_csolve_dw(S.H, S.B, S.H0, S.red, nk);
-    bsync();
+    cluster.sync();
     STAMP(2);
-    // ---- 3. eigenvalues of C: Hessenberg form, then Francis QR on a copy
+    if (!lead) return;
+    // ---- 3. Hessenberg form of C
+    for (int i = tid; i < nk * nk; i += NT) {
+        const int r = i / nk, c = i % nk;
+        S.H[r * LDS + c] = __ldcg(&G->H[r * LDS + c]);
+    }
+    bsync();
     bhessenberg(S.H, S.Vh, S.beta, nk, S.red);
     STAMP(14);
-    for (int i = tid; i < nk * LDS; i += NT) S.H0[i] = S.H[i];
-    if (tid == 0) S.ints[6] = 0;
-    bsync();
-    for (int i = tid; i < kStateWords; i += NT) gst[i] = sst[i];
+    for (int i = tid; i < nk * nk; i += NT) {
+        const int r = i / nk, c = i % nk;
+        G->H0[r * LDS + c] = S.H[r * LDS + c];
+        G->Vh[r * LDS + c] = S.Vh[r * LDS + c];
+    }
+    for (int i = tid; i < nk; i += NT) G->beta[i] = S.beta[i];
 #undef STAMP
 }
 
@@ -838,7 +904,7 @@ __global__ void __launch_bounds__(32) k_eigvec(DenseArgs a) {
     double* sV = sL + MAXM * LDS;
     double* sbeta = sV + MAXM * LDS;
     EigvecDw* E = reinterpret_cast<EigvecDw*>(sbeta + MAXM);
-    const Smem* G = state_of(a);
+    const DenseState* G = state_of(a);
     if (G->ints[6]) return;
     const int u = blockIdx.x;
     const int nsel = G->ints[3], nk = G->ints[0];
@@ -918,7 +984,7 @@ __global__ void __launch_bounds__(32) k_eigvec(DenseArgs a) {
 // are in the diagonal blocks of H (n x n).  Every step takes one thread per
 // eigenvalue, unit or rank (one thread for all of it took 180 us).
 static_assert(kFrancisThreads >= MAXM, "one eigenvalue per thread");
-__device__ void select_units(const DenseArgs& a, Smem* G, const double* H, int n) {
+__device__ void select_units(const DenseArgs& a, DenseState* G, const double* H, int n) {
     __shared__ double er[MAXM], ei[MAXM], ka[MAXM], kr[MAXM];
     __shared__ int slot[MAXM], size[MAXM], order[MAXM], count;
     const int t = threadIdx.x, kp = a.kp;
@@ -990,11 +1056,11 @@ __device__ void select_units(const DenseArgs& a, Smem* G, const double* H, int n
     if (t == 0) G->ints[3] = ns;
 }
 
-// Eigenvalues of the saved Hessenberg form (two warps; see k_extract) and the
+// Eigenvalues of the saved Hessenberg form (two warps; see k_pencil) and the
 // selection.  The stage clocks 3 and 4 and the sweep counts come from this launch.
 __global__ void __launch_bounds__(kFrancisThreads) k_francis(DenseArgs a) {
     extern __shared__ __align__(16) double shh[];
-    Smem* G = state_of(a);
+    DenseState* G = state_of(a);
     if (G->ints[6]) return;
     const int nk = G->ints[0];
     const int t = threadIdx.x;
@@ -1011,7 +1077,7 @@ __global__ void __launch_bounds__(kFrancisThreads) k_francis(DenseArgs a) {
 }
 
 // Two selected units belong to one numerical cluster (u the later one)
-__device__ __forceinline__ bool close_units(const Smem* G, int u, int v) {
+__device__ __forceinline__ bool close_units(const DenseState* G, int u, int v) {
     const int e = G->order[u], f = G->order[v];
     const double mag = fmax(fabs(G->eig_re[e]) + fabs(G->eig_im[e]), 1e-300);
     return fabs(G->eig_re[f] - G->eig_re[e]) + fabs(G->eig_im[f] - G->eig_im[e]) <= 1e-8 * mag;
@@ -1030,7 +1096,7 @@ __global__ void __launch_bounds__(128) k_finish(DenseArgs a) {
     double* R = shy;                  // MAXM x LDS
     double* Y = R + MAXM * LDS;       // [unit][re, im][MAXM]
     __shared__ double rinv[MAXM], W[4][MAXM];
-    const Smem* G = state_of(a);
+    const DenseState* G = state_of(a);
     if (G->ints[6]) return;
     const int nk = G->ints[0], nvk = G->ints[1], nsel = G->ints[3];
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1164,16 +1230,14 @@ __global__ void __launch_bounds__(128) k_finish(DenseArgs a) {
 
 }  // namespace
 
-size_t dense_smem_bytes() { return sizeof(Smem); }
-
 // Yre, Yim (MAXM^2 each; MAXM^2 unused) and the shared-memory state passed
 // between the launches.
 size_t dense_work_doubles() { return kDenseWorkDoubles; }
 static_assert(kWorkMainDoubles >= 3 * (size_t)MAXM * MAXM, "dense scratch layout");
 
 cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
-    size_t shm = sizeof(Smem);
-    cudaError_t e = cudaFuncSetAttribute(k_extract, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    size_t shm = sizeof(PencilShm);
+    cudaError_t e = cudaFuncSetAttribute(k_pencil, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     if (e != cudaSuccess) return e;
     const size_t shf = sizeof(double) * MAXM * LDS;
     e = cudaFuncSetAttribute(k_francis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shf);
@@ -1184,7 +1248,7 @@ cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     const size_t shn = sizeof(double) * (MAXM * LDS + MAXKP * 2 * MAXM);
     e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shn);
     if (e != cudaSuccess) return e;
-    k_extract<<<1, NT, shm, s>>>(a);
+    k_pencil<<<kPencilCtas, NT, shm, s>>>(a);
     k_francis<<<1, kFrancisThreads, shf, s>>>(a);
     k_eigvec<<<a.kp, 32, she, s>>>(a);
     k_finish<<<a.kp, 128, shn, s>>>(a);
@@ -1423,7 +1487,7 @@ extern "C" plhr_status plhr_tharm_extract(int m, int kp, int nv, const double* G
 namespace {
 
 // Scratch of the projected eigensolve for the largest supported basis
-// (m = 64): three 64 x 64 arrays and the saved state, about 263 KiB.  Every
+// (m = 64): three 64 x 64 arrays and the saved state, about 262 KiB.  Every
 // GPU that loads the library holds this array until the process exits.
 constexpr size_t kNoAllocScratchDoubles = plhr::kDenseWorkDoubles;
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];

@@ -29,7 +29,6 @@ struct DenseArgs {
     long long* clk;      // optional: clock64() at stage boundaries (16 entries)
 };
 
-size_t dense_smem_bytes();
 size_t dense_work_doubles();
 cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s);
 
