@@ -173,7 +173,7 @@ __device__ __forceinline__ void warp_solve(const double* Tc, const double* rinv,
 // warp, so that its 16 accesses (odd stride) fall into distinct banks.  One warp
 // forms the reflector's scalars.  Four warps a scheduler hide each other's
 // dependent operations (two threads a column, one warp a scheduler: 522,000 ->
-// HESS_CYC cycles at n = 64).  v and beta describe the same reflector at any
+// 378,000 cycles at n = 64).  v and beta describe the same reflector at any
 // scale, so only H is scaled back; H, Vh and beta are FP64 again on return.
 __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, double* red) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -346,38 +346,68 @@ __device__ __forceinline__ void house3(dw x, dw y, dw z, dw& u1, dw& u2, dw& tau
     beta = dw_mul_pow2(nrm, __fmul_rn(-sg, pow2_inverse_of(sc)));   // sc is a power of two
 }
 
-// (a0 + u1 a1 + u2 a2) tau: the products' leading parts by error-free sums, everything
-// below them in FP32, normalised once
+// (a0 + u1 a1 + u2 a2) tau: the leading parts by error-free sums and products,
+// everything below them in FP32, not normalised (its use, reflected, is a lazily
+// normalised sum)
 __device__ __forceinline__ dw house_dot(dw a0, dw a1, dw a2, dw u1, dw u2, dw tau) {
     const dw p = dw_two_prod(u1.hi, a1.hi), q = dw_two_prod(u2.hi, a2.hi);
     const float lp = __fmaf_rn(u1.hi, a1.lo, __fmaf_rn(u1.lo, a1.hi, p.lo));
     const float lq = __fmaf_rn(u2.hi, a2.lo, __fmaf_rn(u2.lo, a2.hi, q.lo));
     const dw s = dw_two_sum(p.hi, q.hi), v = dw_two_sum(s.hi, a0.hi);
     const float lo = __fadd_rn(__fadd_rn(__fadd_rn(lp, lq), __fadd_rn(s.lo, a0.lo)), v.lo);
-    return dw_mul(dw_two_sum(v.hi, lo), tau);
+    const dw r = dw_two_prod(v.hi, tau.hi);
+    return {r.hi, __fadd_rn(r.lo, __fmaf_rn(lo, tau.hi, __fmul_rn(v.hi, tau.lo)))};
 }
+// a - s u
+__device__ __forceinline__ dw reflected(dw a, dw u, dw s) {
+    dwacc v = dwacc_of(a);
+    dwacc_add_mul(v, dw_neg(s), u);
+    return dwacc_result(v);
+}
+// which ? a : b as two select instructions: a ternary on a value that differs from
+// lane to lane became a branch, with what follows it once per side
+__device__ __forceinline__ dw dw_select(bool which, dw a, dw b) {
+    dw r;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %6, 0;\n\tselp.f32 %0, %2, %4, p;\n\tselp.f32 %1, %3, %5, p;\n\t}"
+        : "=f"(r.hi), "=f"(r.lo)
+        : "f"(a.hi), "f"(a.lo), "f"(b.hi), "f"(b.lo), "r"((int)which));
+    return r;
+}
+// named barriers between the two roles of the iteration: a side that only
+// announces arrives, the other waits
+template <int ID>
+__device__ __forceinline__ void role_arrive() { asm volatile("bar.arrive %0, 96;" ::"n"(ID) : "memory"); }
+template <int ID>
+__device__ __forceinline__ void role_wait() { asm volatile("bar.sync %0, 96;" ::"n"(ID) : "memory"); }
 
 // Francis double-shift QR (Golub & Van Loan Sec. 7.5) on the upper Hessenberg
 // H, eigenvalues only: every transformation is applied to the active window
 // rows/columns l..hi alone (no Schur vectors, no full Schur form), which is
 // all the eigenvalues need.  Deflated 1x1 and 2x2 diagonal blocks remain.
-// kFrancisThreads threads (two warps, on two sub-partitions): in a bulge step
-// each thread updates one column (left reflection) and then one row (right
-// reflection), so a step costs one short double-word chain per side instead of
-// two per lane in one warp; the reflector itself is formed redundantly by
-// every thread.  The iteration runs in double-word arithmetic on H scaled by a
-// power of two to unit norm (H is converted in place: a double and a
-// double-word value take the same 8 bytes) and is converted back at the end.
-// Every entry is updated by the same operations in the same order as with
-// one warp, so the result does not depend on the thread count.  Returns false
-// if the iteration does not converge; sweeps (optional) gets the number of QR
-// sweeps and of bulge steps.
-constexpr int kFrancisThreads = 64;
+//
+// A step's reflector depends on the one before through the 4 x 4 block at the
+// bulge only, so warp 0 chases the bulge alone: it forms the reflector, applies
+// it to the block's columns, then to its rows and to the column that enters the
+// block next (an entry per lane, warp barriers), and reads the next reflector's
+// column.  Two more warps apply the reflector to the remaining columns (left) and
+// rows (right, disjoint from them) while warp 0 forms the next one.  A step costs
+// the chain reflector - left - right on one entry: 980 cycles against 1370
+// with all threads in step, a column and then a row each.
+//
+// The iteration runs in double-word arithmetic on H scaled by a power of two to
+// unit norm (H is converted in place: a double and a double-word value take the
+// same 8 bytes) and is converted back at the end.  Returns false if the iteration
+// does not converge; sweeps (optional) gets the number of QR sweeps and of bulge
+// steps.
+constexpr int kFrancisThreads = 96;   // the named barriers' count
+enum { BAR_REFLECTOR = 1, BAR_APPLIED = 2 };
+constexpr int kFrancisRows = MAXM + 4;   // rows of H in shared memory
 static_assert(kFrancisThreads >= MAXM, "one column / row per thread");
 
-__device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* sweeps) {
+__device__ __forceinline__ bool francis_eigenvalues(double* Hd, int n, long long* sweeps) {
     __shared__ double red[kFrancisThreads / 32];
     __shared__ int last[kFrancisThreads / 32];
+    __shared__ dw refl[2][3];
     const int t = threadIdx.x;
     double anorm = 0.0;
     for (int i = t; i < n * n; i += kFrancisThreads) {
@@ -396,6 +426,9 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
         double v = (c >= r - 1) ? Hd[r * LDS + c] * down : 0.0;
         H[r * LDS + c] = dw_from_double(v);
     }
+    // what the bulge's loads reach beyond the matrix
+    for (int i = t; i < kFrancisRows * LDS; i += kFrancisThreads)
+        if (i >= n * LDS || i % LDS >= n) H[i] = dw_make(0.0f);
     __syncthreads();
     // negligible subdiagonal: relative to the neighbouring diagonal, or to
     // ||H|| (= 1 to 2 after scaling; normwise backward stable).  Only the
@@ -404,7 +437,7 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
     // quickly.  eps is a few units of the double-word precision.
     const float eps = 0x1p-46f;
     const float hnorm = 1.0f;
-    const dw zero = dw_make(0.0f);
+    const dw zero = dw_make(0.0f), one = dw_make(1.0f);
     bool ok = true;
     int hi = n - 1;
     int its = 0, total_its = 0, total_steps = 0;
@@ -472,51 +505,69 @@ __device__ __noinline__ bool francis_eigenvalues(double* Hd, int n, long long* s
         // every thread has read the shift and the first bulge column before
         // any thread writes
         __syncthreads();
-        for (int k = l; k <= hi - 1; ++k) {
-            // rows (columns) k..k+2, the last step's k and k+1 with u2 = 0
-            const bool three = k < hi - 1;
-            // this thread's column of the left reflection (k..hi) is read before the
-            // reflector is formed
-            const int ca = k + t;
-            const bool left = ca <= hi;
-            dw a0 = zero, a1 = zero, a2 = zero;
-            if (left) {
-                a0 = H[k * LDS + ca];
-                a1 = H[(k + 1) * LDS + ca];
-                if (three) a2 = H[(k + 2) * LDS + ca];
+        if (t >= 32) {
+            // reflector k: columns k + 5.. (left), rows ..k - 1 (right); thread q has
+            // column hi - q, then row l + 63 - q (never both: hi - l <= 63)
+            const int q = t - 32, col = hi - q, row = l + 63 - q;
+            for (int k = l; k < hi; ++k) {
+                role_wait<BAR_REFLECTOR>();
+                const bool left = col >= k + 5;
+                if (left || row < k) {
+                    dw* h = H + (left ? k * LDS + col : row * LDS + k);
+                    const int step = left ? LDS : 1;
+                    const dw u1 = refl[k & 1][0], u2 = refl[k & 1][1], tau = refl[k & 1][2];
+                    const dw a0 = h[0], a1 = h[step], a2 = h[2 * step];
+                    const dw sa = house_dot(a0, a1, a2, u1, u2, tau);
+                    h[0] = reflected(a0, one, sa);
+                    h[step] = reflected(a1, u1, sa);
+                    if (k < hi - 1) h[2 * step] = reflected(a2, u2, sa);
+                }
+                if (k < hi - 1) role_arrive<BAR_APPLIED>();
             }
-            dw u1, u2, tau, beta;
-            house3(x, y, three ? z : zero, u1, u2, tau, beta);
-            if (left) {
-                const dw sa = house_dot(a0, a1, a2, u1, u2, tau);
-                H[k * LDS + ca] = dw_sub(a0, sa);
-                H[(k + 1) * LDS + ca] = dw_sub(a1, dw_mul(sa, u1));
-                if (three) H[(k + 2) * LDS + ca] = dw_sub(a2, dw_mul(sa, u2));
-            }
-            __syncthreads();
-            // column k - 1 becomes (beta, 0, 0); every thread has read it above
-            if (k > l && t == kFrancisThreads - 1) {
-                H[k * LDS + k - 1] = beta;
-                H[(k + 1) * LDS + k - 1] = zero;
-                if (three) H[(k + 2) * LDS + k - 1] = zero;
-            }
-            // right: row l + t (rows l..min(k+3, hi))
-            const int ra = l + t;
-            if (ra <= (k + 3 < hi ? k + 3 : hi)) {
-                dw* h = H + ra * LDS + k;
-                const dw b0 = h[0], b1 = h[1], b2 = three ? h[2] : zero;
-                const dw sb = house_dot(b0, b1, b2, u1, u2, tau);
-                h[0] = dw_sub(b0, sb);
-                h[1] = dw_sub(b1, dw_mul(sb, u1));
-                if (three) h[2] = dw_sub(b2, dw_mul(sb, u2));
-            }
-            __syncthreads();
-            if (k < hi - 1) {
+        } else {
+            // lanes 0..11: entry e of column, then row k + c of the block; lanes 12..14
+            // store column k - 1, (beta, 0, 0), then take row k + e of column k + 4;
+            // lanes 16..18 store the reflector.  Every lane loads (the rest of the
+            // last rows is zero or finite, and is not stored), so that nothing but the
+            // stores is conditional.
+            const int c = t & 3, e = t < 12 ? t >> 2 : c;
+            const bool block = t < 12, edge = t >= 12 && t < 15;
+            const dw* from = H + l * LDS + l + c;
+            dw* to = H + (block ? (l + e) * LDS + l + c : (l + e) * LDS + l - 1);
+            dw* rows = H + (block ? (l + c) * LDS + l : l * LDS + l + 4);
+            const int step = block ? 1 : LDS;
+            for (int k = l; k < hi; ++k) {
+                // rows (columns) k..k+2, the last step's k and k+1 with u2 = 0
+                const bool three = k < hi - 1, entry = e < 2 || (e == 2 && three), in = k + c <= hi;
+                const dw a0 = from[0], a1 = from[LDS], a2 = from[2 * LDS];
+                const dw ae = dw_select(e == 0, a0, dw_select(e == 1, a1, a2));
+                dw u1, u2, tau, beta;
+                house3(x, y, three ? z : zero, u1, u2, tau, beta);
+                const dw ue = dw_select(e == 0, one, dw_select(e == 1, u1, u2));
+                const dw va = dw_select(block, reflected(ae, ue, house_dot(a0, a1, a2, u1, u2, tau)),
+                                        dw_select(t == 12, beta, zero));
+                __syncwarp();
+                if (entry && (block ? in : edge && k > l)) *to = va;
+                if (t >= 16 && t < 19) refl[k & 1][c] = dw_select(c == 0, u1, dw_select(c == 1, u2, tau));
+                // the other warps have applied the earlier reflectors to column k + 4
+                if (k > l) role_wait<BAR_APPLIED>();
+                else __syncwarp();
+                const dw b0 = rows[0], b1 = rows[step], b2 = rows[2 * step];
+                const dw be = dw_select(e == 0, b0, dw_select(e == 1, b1, b2));
+                const dw vb = reflected(be, ue, house_dot(b0, b1, b2, u1, u2, tau));
+                __syncwarp();
+                if (entry && (block ? in : edge && k + 4 <= hi)) rows[e * step] = vb;
+                role_arrive<BAR_REFLECTOR>();
+                __syncwarp();
                 x = H[(k + 1) * LDS + k];
                 y = H[(k + 2) * LDS + k];
-                z = (k < hi - 2) ? H[(k + 3) * LDS + k] : zero;
+                z = H[(k + 3) * LDS + k];
+                from += LDS + 1;
+                to += LDS + 1;
+                rows += LDS + 1;
             }
         }
+        __syncthreads();
     }
     __syncthreads();
     for (int i = t; i < n * n; i += kFrancisThreads) {
@@ -674,7 +725,7 @@ __device__ __forceinline__ DenseState* state_of(const DenseArgs& a) {
 }
 
 // The dense stage runs as four launches: k_pencil (up to the Hessenberg form,
-// state saved to global scratch), k_francis (two warps: the eigenvalues and the
+// state saved to global scratch), k_francis (three warps: the eigenvalues and the
 // selection), k_eigvec and k_finish (one CTA per selected unit each: the
 // eigenvector; cluster orthogonalisation, Y' and the coefficients of the unit's
 // columns).  The eigenvalue iteration measured 2x slower per bulge step when run
@@ -1056,7 +1107,7 @@ __device__ void select_units(const DenseArgs& a, DenseState* G, const double* H,
     if (t == 0) G->ints[3] = ns;
 }
 
-// Eigenvalues of the saved Hessenberg form (two warps; see k_pencil) and the
+// Eigenvalues of the saved Hessenberg form (three warps; see k_pencil) and the
 // selection.  The stage clocks 3 and 4 and the sweep counts come from this launch.
 __global__ void __launch_bounds__(kFrancisThreads) k_francis(DenseArgs a) {
     extern __shared__ __align__(16) double shh[];
@@ -1239,7 +1290,7 @@ cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     size_t shm = sizeof(PencilShm);
     cudaError_t e = cudaFuncSetAttribute(k_pencil, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     if (e != cudaSuccess) return e;
-    const size_t shf = sizeof(double) * MAXM * LDS;
+    const size_t shf = sizeof(double) * kFrancisRows * LDS;
     e = cudaFuncSetAttribute(k_francis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shf);
     if (e != cudaSuccess) return e;
     const size_t she = sizeof(double) * kEigvecShmDoubles;
