@@ -591,109 +591,142 @@ __device__ __forceinline__ bool francis_eigenvalues(double* Hd, int n, long long
 struct cdw {
     dw re, im;
 };
-__device__ __forceinline__ cdw cdw_mul(cdw a, cdw b) {
-    return {dw_sub(dw_mul(a.re, b.re), dw_mul(a.im, b.im)), dw_add(dw_mul(a.re, b.im), dw_mul(a.im, b.re))};
+// (products and sums as lazily normalised sums: half the depth of the pairwise ones)
+__device__ __forceinline__ cdw cdw_fma(cdw c, cdw a, cdw b) {   // c + a b
+    dwacc r = dwacc_of(c.re), i = dwacc_of(c.im);
+    dwacc_add_mul(r, a.re, b.re);
+    dwacc_add_mul(r, dw_neg(a.im), b.im);
+    dwacc_add_mul(i, a.re, b.im);
+    dwacc_add_mul(i, a.im, b.re);
+    return {dwacc_result(r), dwacc_result(i)};
 }
-__device__ __forceinline__ cdw cdw_sub(cdw a, cdw b) { return {dw_sub(a.re, b.re), dw_sub(a.im, b.im)}; }
+__device__ __forceinline__ cdw cdw_zero() { return {dw_make(0.0f), dw_make(0.0f)}; }
+__device__ __forceinline__ cdw cdw_mul(cdw a, cdw b) { return cdw_fma(cdw_zero(), a, b); }
+__device__ __forceinline__ cdw cdw_neg(cdw a) { return {dw_neg(a.re), dw_neg(a.im)}; }
+__device__ __forceinline__ dw dw_fma(dw c, dw a, dw b) {   // c + a b
+    dwacc r = dwacc_of(c);
+    dwacc_add_mul(r, a, b);
+    return dwacc_result(r);
+}
 __device__ __forceinline__ float cdw_abs1(cdw a) { return fabsf(a.re.hi) + fabsf(a.im.hi); }
 // 1 / b, the denominator scaled by a power of two first (no under- or overflow)
 __device__ __forceinline__ cdw cdw_recip(cdw b) {
     const float sc = pow2_inverse_of(fmaxf(fabsf(b.re.hi), fabsf(b.im.hi)));
     const dw r = dw_mul_pow2(b.re, sc), i = dw_mul_pow2(b.im, sc);
-    const dw den = dw_add(dw_mul(r, r), dw_mul(i, i));
-    const dw inv = dw_div(dw_make(1.0f), den);
+    const dw den = dw_fma(dw_fma(dw_make(0.0f), r, r), i, i);
+    const dw inv = recip_refine(den, __fdividef(1.0f, den.hi));
     return {dw_mul_pow2(dw_mul(r, inv), sc), dw_mul_pow2(dw_neg(dw_mul(i, inv)), sc)};
 }
+__device__ __forceinline__ dw dw_shfl(dw v, int lane) {
+    return {__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
+}
+__device__ __forceinline__ cdw cdw_shfl(cdw v, int lane) { return {dw_shfl(v.re, lane), dw_shfl(v.im, lane)}; }
 
-// Inverse iteration on the Hessenberg H0 (FP64, scaled here by `down`, a power
-// of two) for the eigenvalue lam (same scale): (H0 - lam I) is factored once
-// by Gaussian elimination with adjacent-row pivoting (keeps the Hessenberg
-// structure; multipliers, swaps, the packed upper factor U and the
-// reciprocals of its pivots kept), then two solves starting from b = 1, each
-// normalised to max |x_i| = 1.  Column-oriented back substitution: one
-// reciprocal multiply on the critical path per step, the updates in parallel.
+// A vector or matrix row over a warp: entries lane and lane + 32
+struct cdw2 {
+    cdw v[2];
+    __device__ __forceinline__ cdw at(int j) const { return cdw_shfl(j >= 32 ? v[1] : v[0], j & 31); }
+};
 
-__device__ void inverse_iteration_dw(const double* H0, int n, double down, cdw lam, cdw* x, cdw* U, cdw* mult,
-                                     cdw* rpiv, int* swp, cdw* cur, cdw* nxt, float tiny) {
+// Inverse iteration on the Hessenberg H (n x n, unit norm) for the eigenvalue lam
+// by one warp: (H - lam I) is factored once by Gaussian elimination with
+// adjacent-row pivoting (keeps the Hessenberg structure; multipliers, swaps, the
+// upper factor U and the reciprocals of its pivots kept), then two solves starting
+// from b = 1, each normalised to max |x_i| = 1.  The row being eliminated and the
+// vector stay in registers; U and the multipliers go to shared memory.
+// Column-oriented back substitution: one reciprocal multiply on the critical path
+// per step, the updates in parallel.
+__device__ cdw2 inverse_iteration(const dw* H, int n, cdw lam, cdw* U, cdw* mult, cdw* rpiv, cdw* xs, int* swp,
+                                  float tiny) {
     const int lane = threadIdx.x & 31;
-    const cdw zero = {dw_make(0.0f), dw_make(0.0f)};
-    auto hs = [&](int r, int c) -> cdw {
-        dw v = dw_from_double(H0[r * LDS + c] * down);
-        cdw e = {v, dw_make(0.0f)};
-        if (r == c) e = cdw_sub(e, lam);
-        return e;
-    };
-    for (int j = lane; j < n; j += 32) cur[j] = hs(0, j);
-    wsync();
-    for (int k = 0; k < n - 1; ++k) {
-        for (int j = k + lane; j < n; j += 32) nxt[j] = (j >= k) ? hs(k + 1, j) : zero;
-        wsync();
-        const bool swap = cdw_abs1(nxt[k]) > cdw_abs1(cur[k]);
-        wsync();
+    cdw2 cur, nxt;
+    for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        cur.v[q] = {j < n ? H[j] : dw_make(0.0f), dw_make(0.0f)};
+        if (j == 0) cur.v[q] = {dw_sub(cur.v[q].re, lam.re), dw_neg(lam.im)};
+    }
+    for (int k = 0; k < n; ++k) {
+        cdw piv = cur.at(k);
+        if (k < n - 1) {
+            for (int q = 0; q < 2; ++q) {
+                const int j = lane + 32 * q;
+                nxt.v[q] = {j >= k && j < n ? H[(k + 1) * LDS + j] : dw_make(0.0f), dw_make(0.0f)};
+                if (j == k + 1) nxt.v[q] = {dw_sub(nxt.v[q].re, lam.re), dw_neg(lam.im)};
+            }
+        }
+        cdw low = {k < n - 1 ? H[(k + 1) * LDS + k] : dw_make(0.0f), dw_make(0.0f)};
+        const bool swap = k < n - 1 && cdw_abs1(low) > cdw_abs1(piv);
         if (swap) {
-            for (int j = k + lane; j < n; j += 32) { const cdw t2 = cur[j]; cur[j] = nxt[j]; nxt[j] = t2; }
+            const cdw2 t = cur;
+            cur = nxt;
+            nxt = t;
+            const cdw u = piv;
+            piv = low;
+            low = u;
         }
-        wsync();
-        cdw piv = cur[k];
         if (cdw_abs1(piv) < tiny) piv = {dw_make(tiny), dw_make(0.0f)};
-        const cdw rp = cdw_recip(piv);
-        const cdw f = cdw_mul(nxt[k], rp);
-        cdw* urow = U + (k * n - (k * (k - 1)) / 2);   // row k holds columns k..n-1
-        for (int j = k + lane; j < n; j += 32) {
-            urow[j - k] = (j == k) ? piv : cur[j];
-            if (j > k) nxt[j] = cdw_sub(nxt[j], cdw_mul(f, cur[j]));
+        const cdw rp = cdw_recip(piv), f = cdw_mul(low, rp), nf = cdw_neg(f);
+        for (int q = 0; q < 2; ++q) {
+            const int j = lane + 32 * q;
+            if (j < n && j >= k) U[k * LDS + j] = j == k ? piv : cur.v[q];
+            cur.v[q] = cdw_fma(nxt.v[q], nf, cur.v[q]);   // the next row (columns above k)
         }
-        if (lane == 0) { mult[k] = f; rpiv[k] = rp; swp[k] = swap ? 1 : 0; }
-        wsync();
-        for (int j = k + 1 + lane; j < n; j += 32) cur[j] = nxt[j];
-        wsync();
+        if (lane == 0) { mult[k] = nf; rpiv[k] = rp; swp[k] = swap ? 1 : 0; }
     }
-    {
-        cdw piv = cur[n - 1];
-        if (cdw_abs1(piv) < tiny) piv = {dw_make(tiny), dw_make(0.0f)};
-        if (lane == 0) {
-            U[(n - 1) * n - ((n - 1) * (n - 2)) / 2] = piv;
-            rpiv[n - 1] = cdw_recip(piv);
-        }
-    }
-    for (int i = lane; i < n; i += 32) x[i] = {dw_make(1.0f), dw_make(0.0f)};
+    cdw2 x;
+    x.v[0] = x.v[1] = {dw_make(1.0f), dw_make(0.0f)};
     wsync();
     for (int iter = 0; iter < 2; ++iter) {
-        // forward: the recorded row swaps and eliminations applied to b = x
-        if (lane == 0) {
-            for (int k = 0; k < n - 1; ++k) {
-                if (swp[k]) { const cdw t2 = x[k]; x[k] = x[k + 1]; x[k + 1] = t2; }
-                x[k + 1] = cdw_sub(x[k + 1], cdw_mul(mult[k], x[k]));
-            }
-        }
+        // forward: the recorded row swaps and eliminations applied to b = x, one
+        // chain that every lane follows
+        for (int q = 0; q < 2; ++q)
+            if (lane + 32 * q < n) xs[lane + 32 * q] = x.v[q];
         wsync();
+        cdw top = xs[0];
+        for (int k = 0; k < n - 1; ++k) {
+            const cdw nf = mult[k];
+            cdw next = xs[k + 1];
+            if (swp[k]) {
+                const cdw t = top;
+                top = next;
+                next = t;
+            }
+            if (k == lane) x.v[0] = top;
+            if (k == lane + 32) x.v[1] = top;
+            top = cdw_fma(next, nf, top);
+        }
+        if (n - 1 == lane) x.v[0] = top;
+        if (n - 1 == lane + 32) x.v[1] = top;
         // backward: x_i = b_i / U_ii, then b_j -= U_ji x_i for j < i
         for (int i = n - 1; i >= 0; --i) {
-            const cdw xi_ = cdw_mul(x[i], rpiv[i]);
-            wsync();
-            for (int j = lane; j < i; j += 32) {
-                const cdw u = U[j * n - (j * (j - 1)) / 2 + (i - j)];
-                x[j] = cdw_sub(x[j], cdw_mul(u, xi_));
+            const cdw xi = cdw_mul(x.at(i), rpiv[i]), ni = cdw_neg(xi);
+            if (lane < i) x.v[0] = cdw_fma(x.v[0], U[lane * LDS + i], ni);
+            if (i > 32) {
+                if (lane + 32 < i) x.v[1] = cdw_fma(x.v[1], U[(lane + 32) * LDS + i], ni);
             }
-            if (lane == 0) x[i] = xi_;
-            wsync();
+            if (lane == i) x.v[0] = xi;
+            if (lane + 32 == i) x.v[1] = xi;
         }
         // normalise to max |x_i| = 1 (scale by a power of two, then exactly)
         float mx = 0.0f;
-        for (int j = lane; j < n; j += 32) mx = fmaxf(mx, cdw_abs1(x[j]));
+        for (int q = 0; q < 2; ++q)
+            if (lane + 32 * q < n) mx = fmaxf(mx, cdw_abs1(x.v[q]));
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const float sc = (mx > 0.0f && isfinite(mx)) ? pow2_inverse_of(mx) : 1.0f;
-        for (int j = lane; j < n; j += 32) x[j] = {dw_mul_pow2(x[j].re, sc), dw_mul_pow2(x[j].im, sc)};
+        for (int q = 0; q < 2; ++q) x.v[q] = {dw_mul_pow2(x.v[q].re, sc), dw_mul_pow2(x.v[q].im, sc)};
         wsync();
     }
+    return x;
 }
 
-__device__ __forceinline__ dw warp_sum_dw(dw v) {
+// sum over the warp, lazily normalised
+__device__ __forceinline__ dw warp_sum_dw(dwacc v) {
     for (int o = 16; o > 0; o >>= 1) {
-        const dw t = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-        v = dw_add(v, t);
+        const float h = __shfl_xor_sync(0xffffffffu, v.hi, o), l = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        const dw t = dw_two_sum(v.hi, h);
+        v = {t.hi, __fadd_rn(t.lo, __fadd_rn(v.lo, l))};
     }
-    return v;
+    return dwacc_result(v);
 }
 
 // ---------------------------------------------------------------- the state between the launches
@@ -713,10 +746,8 @@ struct DenseState {
     int ints[8];              // [0] kept columns, [1] of V, [3] selected units, [6] stop, [7] pencil's verdict
 };
 
-// Yre, Yim (MAXM^2 each; MAXM^2 unused), then the saved state; a selected unit (at most
-// MAXKP) keeps its packed complex LU factor (MAXM (MAXM+1) / 2) in shared memory
+// Yre, Yim (MAXM^2 each; MAXM^2 unused), then the saved state
 constexpr int MAXKP = 16;
-constexpr size_t kLuComplex = (size_t)MAXM * (MAXM + 1) / 2;
 constexpr size_t kWorkMainDoubles = 3 * (size_t)MAXM * MAXM;
 constexpr size_t kDenseWorkDoubles = kWorkMainDoubles + (sizeof(DenseState) + sizeof(double) - 1) / sizeof(double);
 
@@ -932,102 +963,100 @@ __global__ void __cluster_dims__(kPencilCtas, 1, 1) __launch_bounds__(NT) k_penc
 #undef STAMP
 }
 
-// Eigenvector of one selected unit (CTA u, one warp): inverse iteration on the
-// saved Hessenberg form H0, back to C's basis with the Householder reflectors,
-// then y = L^{-T} z in the orthonormal basis, into Yre[u], Yim[u].  The units
-// run as separate CTAs on separate SMs (the FP64 work of one unit is serial).
-// shared memory of k_eigvec: H0, the Cholesky factor L of G_L and the
-// Householder vectors (MAXM x LDS each), the reflector coefficients, then the
-// double-word working set: the packed LU factor of the inverse iteration,
-// its multipliers, pivot reciprocals and row swaps, the vector and two work
-// rows, and the result y (re, im)
-struct EigvecDw {
-    cdw U[kLuComplex];
-    cdw mult[MAXM], rpiv[MAXM], x[MAXM], cur[MAXM], nxt[MAXM];
-    dw yr[MAXM], yi[MAXM];
-    int swp[MAXM];
+// Eigenvector of one selected unit (CTA u): inverse iteration on the saved
+// Hessenberg form H0, back to C's basis with the Householder reflectors, then
+// y = L^{-T} z in the orthonormal basis, into Yre[u], Yim[u].  The units run as
+// separate CTAs on separate SMs; one warp follows a unit's serial chain, after all
+// four have brought the three matrices to double-word form (in the chain, the
+// conversions and a division per row of L were 40 % of it).  250 -> 140 us at
+// m = 64.
+struct EigvecShm {
+    dw H[MAXM * LDS], L[MAXM * LDS], V[MAXM * LDS];
+    cdw U[MAXM * LDS];
+    cdw mult[MAXM], rpiv[MAXM], x[MAXM];
+    dw beta[MAXM], rl[MAXM];
+    int swp[MAXM], top[2];
 };
-constexpr size_t kEigvecShmDoubles = 3 * (size_t)MAXM * LDS + MAXM + (sizeof(EigvecDw) + 7) / 8;
 
-__global__ void __launch_bounds__(32) k_eigvec(DenseArgs a) {
-    extern __shared__ __align__(16) double sh0[];
-    double* sL = sh0 + MAXM * LDS;
-    double* sV = sL + MAXM * LDS;
-    double* sbeta = sV + MAXM * LDS;
-    EigvecDw* E = reinterpret_cast<EigvecDw*>(sbeta + MAXM);
+// 2^-k for the largest exponent k of a matrix, from the upper words of its entries
+__device__ __forceinline__ double unit_scale(int top) {
+    return top < 0x00100000 ? 1.0 : ldexp(1.0, 1023 - (top >> 20));
+}
+
+__global__ void __launch_bounds__(128) k_eigvec(DenseArgs a) {
+    extern __shared__ __align__(16) unsigned char she[];
+    EigvecShm& S = *reinterpret_cast<EigvecShm*>(she);
     const DenseState* G = state_of(a);
     if (G->ints[6]) return;
-    const int u = blockIdx.x;
-    const int nsel = G->ints[3], nk = G->ints[0];
+    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const int nsel = G->ints[3], n = G->ints[0];
     if (u >= nsel) return;
-    const int lane = threadIdx.x;
-    double hn = 0.0, ln = 0.0;
-    for (int i = lane; i < nk * LDS; i += 32) {
-        const double v = G->H0[i];
-        sh0[i] = v;
-        sL[i] = G->B[i];
-        sV[i] = G->Vh[i];
-        if (i % LDS < nk) {
-            hn = fmax(hn, fabs(v));
-            ln = fmax(ln, fabs(G->B[i]));
-        }
+    if (tid < 2) S.top[tid] = 0;
+    __syncthreads();
+    int th = 0, tl = 0;
+    for (int i = tid; i < n * LDS; i += 128) {
+        if (i % LDS >= n) continue;
+        th = max(th, __double2hiint(G->H0[i]) & 0x7fffffff);
+        tl = max(tl, __double2hiint(G->B[i]) & 0x7fffffff);
     }
-    for (int i = lane; i < nk; i += 32) sbeta[i] = G->beta[i];
-    hn = warp_max(hn);
-    ln = warp_max(ln);
-    __syncwarp();
-    // H0 and lam scaled by a power of two to unit norm
-    const double down = ldexp(1.0, -(hn > 0.0 ? ilogb(hn) : 0));
+    atomicMax(&S.top[0], th);
+    atomicMax(&S.top[1], tl);
+    __syncthreads();
+    // H0 and lam, and L, scaled by a power of two to unit norm
+    const double down = unit_scale(S.top[0]), ld = unit_scale(S.top[1]);
+    for (int i = tid; i < n * LDS; i += 128) {
+        if (i % LDS >= n) continue;
+        S.H[i] = dw_from_double_fast(G->H0[i] * down);
+        S.L[i] = dw_from_double_fast(G->B[i] * ld);
+        if (i < (n - 2) * LDS) S.V[i] = dw_from_double_fast(G->Vh[i]);
+    }
+    if (tid < n) {
+        if (tid < n - 2) S.beta[tid] = dw_from_double_fast(G->beta[tid]);
+        S.rl[tid] = dw_div(dw_make(1.0f), dw_from_double_fast(G->B[tid * LDS + tid] * ld));
+    }
+    __syncthreads();
+    if (tid >= 32) return;
     const int e = G->order[u];
     double lre = G->eig_re[e], lim = G->eig_im[e];
     if (G->nclose[u] > 0) { lre *= 1.0 + 1e-10 * G->nclose[u]; lim *= 1.0 + 1e-10 * G->nclose[u]; }
     const cdw lam = {dw_from_double(lre * down), dw_from_double(lim * down)};
     const float tiny = 0x1p-46f;   // a few units of the double-word precision of the unit-norm matrix
-    inverse_iteration_dw(sh0, nk, down, lam, E->x, E->U, E->mult, E->rpiv, E->swp, E->cur, E->nxt, tiny);
+    cdw2 x = inverse_iteration(S.H, n, lam, S.U, S.mult, S.rpiv, S.x, S.swp, tiny);
     // z = Q x with Q = H_0 H_1 ... (reflectors applied last-first)
-    for (int k = nk - 3; k >= 0; --k) {
-        const double bk = sbeta[k];
-        if (bk == 0.0) continue;
-        const double* v = sV + k * LDS;
-        dw sr = dw_make(0.0f), si = dw_make(0.0f);
-        for (int i = k + 1 + lane; i < nk; i += 32) {
-            const dw vi = dw_from_double(v[i]);
-            sr = dw_add(sr, dw_mul(vi, E->x[i].re));
-            si = dw_add(si, dw_mul(vi, E->x[i].im));
+    for (int k = n - 3; k >= 0; --k) {
+        dw v[2];
+        dwacc sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
+        for (int q = 0; q < 2; ++q) {
+            const int j = lane + 32 * q;
+            v[q] = j < n ? S.V[k * LDS + j] : dw_make(0.0f);
+            dwacc_add_mul(sr, v[q], x.v[q].re);
+            dwacc_add_mul(si, v[q], x.v[q].im);
         }
-        const dw b = dw_from_double(bk);
-        sr = dw_mul(warp_sum_dw(sr), b);
-        si = dw_mul(warp_sum_dw(si), b);
-        __syncwarp();
-        for (int i = k + 1 + lane; i < nk; i += 32) {
-            const dw vi = dw_from_double(v[i]);
-            E->x[i].re = dw_sub(E->x[i].re, dw_mul(sr, vi));
-            E->x[i].im = dw_sub(E->x[i].im, dw_mul(si, vi));
-        }
-        __syncwarp();
+        const dw b = dw_neg(S.beta[k]);
+        const dw tr = dw_mul(warp_sum_dw(sr), b), ti = dw_mul(warp_sum_dw(si), b);
+        for (int q = 0; q < 2; ++q) x.v[q] = {dw_fma(x.v[q].re, v[q], tr), dw_fma(x.v[q].im, v[q], ti)};
     }
     // y = L^{-T} z: column-oriented back substitution with the lower factor L
     // (scaled to unit norm; y then carries the inverse scale, undone below)
-    const double ld = ldexp(1.0, -(ln > 0.0 ? ilogb(ln) : 0));
-    for (int i = lane; i < nk; i += 32) { E->yr[i] = E->x[i].re; E->yi[i] = E->x[i].im; }
-    __syncwarp();
-    for (int i = nk - 1; i >= 0; --i) {
-        const dw rl = dw_div(dw_make(1.0f), dw_from_double(sL[i * LDS + i] * ld));
-        const dw yr = dw_mul(E->yr[i], rl), yi = dw_mul(E->yi[i], rl);
-        __syncwarp();
-        for (int j = lane; j < i; j += 32) {
-            const dw l = dw_from_double(sL[i * LDS + j] * ld);
-            E->yr[j] = dw_sub(E->yr[j], dw_mul(l, yr));
-            E->yi[j] = dw_sub(E->yi[j], dw_mul(l, yi));
+    for (int i = n - 1; i >= 0; --i) {
+        const cdw t = x.at(i);
+        const dw rl = S.rl[i];
+        const dw yr = dw_mul(t.re, rl), yi = dw_mul(t.im, rl);
+        for (int q = 0; q < 2; ++q) {
+            const int j = lane + 32 * q;
+            if (q == 1 && i <= 32 && i != j) continue;
+            const dw l = j < i ? S.L[i * LDS + j] : dw_make(0.0f);
+            if (j < i) x.v[q] = {dw_fma(x.v[q].re, l, dw_neg(yr)), dw_fma(x.v[q].im, l, dw_neg(yi))};
+            if (j == i) x.v[q] = {yr, yi};
         }
-        if (lane == 0) { E->yr[i] = yr; E->yi[i] = yi; }
-        __syncwarp();
     }
     double* yr = a.work + (size_t)u * MAXM;
     double* yi = a.work + (size_t)MAXM * MAXM + (size_t)u * MAXM;
-    for (int i = lane; i < nk; i += 32) {
-        yr[i] = dw_to_double(E->yr[i]) * ld;
-        yi[i] = dw_to_double(E->yi[i]) * ld;
+    for (int q = 0; q < 2; ++q) {
+        const int i = lane + 32 * q;
+        if (i >= n) break;
+        yr[i] = dw_to_double(x.v[q].re) * ld;
+        yi[i] = dw_to_double(x.v[q].im) * ld;
     }
 }
 
@@ -1293,7 +1322,7 @@ cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     const size_t shf = sizeof(double) * kFrancisRows * LDS;
     e = cudaFuncSetAttribute(k_francis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shf);
     if (e != cudaSuccess) return e;
-    const size_t she = sizeof(double) * kEigvecShmDoubles;
+    const size_t she = sizeof(EigvecShm);
     e = cudaFuncSetAttribute(k_eigvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she);
     if (e != cudaSuccess) return e;
     const size_t shn = sizeof(double) * (MAXM * LDS + MAXKP * 2 * MAXM);
@@ -1301,7 +1330,7 @@ cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     k_pencil<<<kPencilCtas, NT, shm, s>>>(a);
     k_francis<<<1, kFrancisThreads, shf, s>>>(a);
-    k_eigvec<<<a.kp, 32, she, s>>>(a);
+    k_eigvec<<<a.kp, 128, she, s>>>(a);
     k_finish<<<a.kp, 128, shn, s>>>(a);
     count_launches(4);
     return cudaGetLastError();
