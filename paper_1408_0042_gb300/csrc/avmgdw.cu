@@ -306,6 +306,65 @@ __global__ void __launch_bounds__(kT) k_restrict_line(Ld gf, Ld gc, int lin, con
     }
 }
 
+// Linear restriction in 3D, four coarse lines (2 along y x 2 along z) per CTA: a fine
+// value is read 2.25 times instead of 4, six independent loads at a time instead of
+// one after the other.  The weights are 1 and 3, the power of two comes last
+// (96 x 80 x 64 x 16: 69 -> 27 us).
+constexpr int kQuadT = 512;
+constexpr size_t kQuadSmemMax = 96 * 1024;
+__global__ void __launch_bounds__(kQuadT) k_restrict_quad(Ld gf, Ld gc, const dw* __restrict__ f,
+                                                          dw* __restrict__ rc) {
+    extern __shared__ dw qsh[];   // [z][y][fine x][column]
+    const int y0 = 4 * blockIdx.x - 1, z0 = 4 * blockIdx.y - 1, nc = gf.nc, line = gf.nx * nc;
+    auto add = [](dwacc& s, dw v, float w) {
+        if (w == 1.0f) dwacc_add(s, v);
+        else dwacc_add_mul_f(s, v, w);
+    };
+    for (int t = threadIdx.x; t < line; t += kQuadT) {
+        dwacc acc[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[o] = {0.0f, 0.0f};
+        const dw* p = f + ((int64_t)z0 * gf.ny + y0) * line + t;
+#pragma unroll 1
+        for (int a = 0; a < 6; ++a, p += (int64_t)gf.ny * line) {
+            if (z0 + a < 0 || z0 + a >= gf.nz) continue;
+            dw v[6];
+#pragma unroll
+            for (int b = 0; b < 6; ++b)
+                v[b] = y0 + b >= 0 && y0 + b < gf.ny ? p[(int64_t)b * line] : dw_make(0.0f);
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {   // the two coarse lines of the plane
+                dwacc s = dwacc_of(v[2 * o]);
+                dwacc_add(s, v[2 * o + 3]);
+                dwacc_add_mul_f(s, v[2 * o + 1], 3.0f);
+                dwacc_add_mul_f(s, v[2 * o + 2], 3.0f);
+                const dw y = dwacc_result(s);
+                if (a < 4) add(acc[o], y, a == 1 || a == 2 ? 3.0f : 1.0f);
+                if (a > 1) add(acc[2 + o], y, a == 3 || a == 4 ? 3.0f : 1.0f);
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) qsh[o * line + t] = dwacc_result(acc[o]);
+    }
+    __syncthreads();
+    for (int o = 0; o < 4; ++o) {
+        const int Y = 2 * blockIdx.x + (o & 1), Z = 2 * blockIdx.y + (o >> 1);
+        if (Y >= gc.ny || Z >= gc.nz) continue;
+        const dw* s = qsh + o * line;
+        dw* dst = rc + ((int64_t)Z * gc.ny + Y) * gc.nx * nc;
+        for (int t = threadIdx.x; t < gc.nx * nc; t += kQuadT) {
+            const int X = t / nc;
+            const dw* q = s + 2 * X * nc + (t - X * nc);
+            dwacc acc = {0.0f, 0.0f};
+            dwacc_add_mul_f(acc, q[0], 3.0f);
+            dwacc_add_mul_f(acc, q[nc], 3.0f);
+            if (X > 0) dwacc_add(acc, q[-nc]);
+            if (2 * X + 2 < gf.nx) dwacc_add(acc, q[2 * nc]);
+            dst[t] = dw_mul_pow2(dwacc_result(acc), 1.0f / 512.0f);
+        }
+    }
+}
+
 // the line kernels keep one x-line of all columns in shared memory
 constexpr size_t kLineSmemMax = 48 * 1024;
 
@@ -489,7 +548,16 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, co
         PLHR_LD(k_shifted, gr, g, sig, cur, bf.tmp);
         PLHR_LD(k_poly, gr, g, sig, dw_host(L.c * L.c), dw_host(0.5 / L.c), om, 1, cur, bf.tmp, r, nxt);
     }
-    if (sizeof(dw) * L.g.nx * nc <= kLineSmemMax && Lc.g.ny <= 65535 && Lc.g.nz <= 65535) {
+    const size_t quad = 4 * sizeof(dw) * L.g.nx * nc;
+    cudaError_t e;
+    if (d3 && H.linear && quad <= kQuadSmemMax && Lc.g.nz <= 65535 && L.g.nx * nc >= kQuadT &&
+        ((Lc.g.ny + 1) / 2) * ((Lc.g.nz + 1) / 2) >= sm_count()) {
+        e = cudaFuncSetAttribute(k_restrict_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQuadSmemMax);
+        if (e != cudaSuccess) return e;
+        k_restrict_quad<<<dim3((unsigned)((Lc.g.ny + 1) / 2), (unsigned)((Lc.g.nz + 1) / 2)), kQuadT, quad, s>>>(
+            g, gc, nxt, bf.rc);
+        count_launches(1);
+    } else if (sizeof(dw) * L.g.nx * nc <= kLineSmemMax && Lc.g.ny <= 65535 && Lc.g.nz <= 65535) {
         const dim3 gl((unsigned)Lc.g.ny, (unsigned)Lc.g.nz);
         const size_t sh = sizeof(dw) * L.g.nx * nc;
         if (d3) k_restrict_line<true><<<gl, kT, sh, s>>>(g, gc, H.linear, nxt, bf.rc);
@@ -498,7 +566,7 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, co
     } else {
         PLHR_LD(k_restrict, grc, g, gc, H.linear, nxt, bf.rc);
     }
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = vcycle(H, l - 1, nc, bf.rc, bf.wc, B, s);
     if (e != cudaSuccess) return e;
