@@ -23,6 +23,7 @@ struct Ld {
 
 struct CoarseDw {
     using V = dw;
+    static constexpr int kLeast = 400;   // V-cycles with 216 points 52 us against 54, with 8^3 42 against 40
     static __device__ __forceinline__ V zero() { return dw_make(0.0f); }
     static __device__ __forceinline__ void madd(V& s, V a, V b) { s = dw_add(s, dw_mul(a, b)); }
     static __device__ __forceinline__ V scale(V x, V mx, V my, V mz, V sig, int) {

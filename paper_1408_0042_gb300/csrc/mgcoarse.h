@@ -21,6 +21,7 @@ namespace plhr {
 // Arithmetic of a form: V values, Vs the basis and eigenvalue entries
 struct CoarseF64 {
     using V = double;
+    static constexpr int kLeast = 0;   // points from which the three kernels win
     static __device__ __forceinline__ V zero() { return 0.0; }
     static __device__ __forceinline__ void madd(V& s, V a, V b) { s += a * b; }
     static __device__ __forceinline__ V scale(V x, V mx, V my, V mz, V sig, int signed_inv) {
@@ -30,6 +31,7 @@ struct CoarseF64 {
 };
 struct CoarseF32 {
     using V = float;
+    static constexpr int kLeast = 600;   // V-cycles with 8^3 points 34 us against 36, with 14 x 10 x 6 equal
     static __device__ __forceinline__ V zero() { return 0.0f; }
     static __device__ __forceinline__ void madd(V& s, V a, V b) { s += a * b; }
     static __device__ __forceinline__ V scale(V x, V mx, V my, V mz, V sig, int) {
@@ -131,11 +133,11 @@ template <class A>
 size_t coarse_line_smem(const Grid& g) {
     return sizeof(typename A::V) * (size_t)(2 * g.nz * kCoarseLine + g.nz * g.nz);
 }
-// whether the three kernels take this grid: 3D, a plane and a bundle of z-lines
+// whether the three kernels take this grid: 3D, large enough that three launches pay, a plane and a bundle of z-lines
 // fit shared memory, 32-bit launch sizes
 template <class A>
 bool coarse_split(const Grid& g, int nc) {
-    return g.d == 3 && g.nx <= 1024 && g.ny <= 1024 && g.nz <= 1024 && coarse_plane_smem<A>(g) <= kCoarseSmem &&
+    return g.d == 3 && g.n() >= A::kLeast && g.nx <= 1024 && g.ny <= 1024 && g.nz <= 1024 && coarse_plane_smem<A>(g) <= kCoarseSmem &&
            coarse_line_smem<A>(g) <= kCoarseSmem && g.nz * (int64_t)nc < (1 << 30) &&
            g.nx * g.ny * (int64_t)nc < ((int64_t)1 << 35);
 }
