@@ -99,41 +99,52 @@ __device__ __forceinline__ void sqrt_and_inverse(double p, double& r, double& ri
 // Cholesky A = R^T R of a symmetric n x n (upper triangle used and replaced).
 // With keep, column j is dropped when its pivot is below tol (the matrix is
 // column-normalised, so the test is relative); without, a pivot that is not
-// above tol ends it (false).  Two warps on two sub-partitions form the pivot's
-// root and scale the row (one product and a correction with the remainder instead
-// of a division an entry), all warps update: the chain of a column is about 13
-// FP64 operations (64 columns: 291,000 -> 208,000 cycles).
+// above tol ends it (false).  Warps 0 and 1, on two sub-partitions, bring row
+// j + 1 up to date, form its pivot's root and scale it (a product and a correction
+// with the remainder instead of a division an entry) while the warps of the other
+// two sub-partitions update the rows below with row j: a column is the longer of a
+// chain of about 14 FP64 operations and the update, and one barrier (64 columns
+// with the Gram's normalisation: 291,000 -> 133,000 cycles).
 __device__ bool bchol(double* A, int n, int* keep, double tol) {
-    const int tid = threadIdx.x;
-    for (int j = 0; j < n; ++j) {
-        const double p = A[j * LDS + j];
-        const bool ok = (p > tol) && isfinite(p);
-        if (!ok && !keep) {
-            bsync();
-            return false;
-        }
-        double r = 0.0;
-        if (ok && tid < 64) {
-            double ri;
-            sqrt_and_inverse(p, r, ri);
-            const int l = j + 1 + tid;
-            if (l < n) {
-                const double v = A[j * LDS + l], q = v * ri;
-                A[j * LDS + l] = fma(fma(-q, r, v), ri, q);
+    __shared__ int stop[2];   // by parity: a thread may read its entry while the next is written
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int ut = (warp >> 2) * 64 + (warp & 1) * 32 + (tid & 31);   // of warps 2, 3 mod 4
+    if (tid < 2) stop[tid] = 0;
+    bsync();
+    double root = 0.0;   // thread 0: the last row's diagonal entry, written one barrier later
+    for (int j = -1; j < n; ++j) {
+        if (tid < 64) {
+            if (tid == 0 && j >= 0) A[j * LDS + j] = root;
+            const int i = j + 1, l = i + tid;
+            if (i < n) {
+                const double f = j >= 0 ? A[j * LDS + i] : 0.0;
+                const double p = fma(-f, f, A[i * LDS + i]);
+                const bool ok = (p > tol) && isfinite(p);
+                double v = 0.0;
+                if (l < n) v = fma(-f, j >= 0 ? A[j * LDS + l] : 0.0, A[i * LDS + l]);
+                root = 0.0;
+                if (ok) {
+                    double ri;
+                    sqrt_and_inverse(p, root, ri);
+                    const double q = v * ri;
+                    v = fma(fma(-q, root, v), ri, q);
+                } else {
+                    v = 0.0;
+                }
+                if (tid > 0 && l < n) A[i * LDS + l] = v;
+                if (tid == 0) {
+                    if (keep) keep[i] = ok ? 1 : 0;
+                    else if (!ok) stop[i & 1] = 1;
+                }
             }
-        }
-        bsync();
-        if (keep && tid == 0) keep[j] = ok ? 1 : 0;
-        if (ok) {
-            if (tid == 0) A[j * LDS + j] = r;
-            for (int a = j + 1 + (tid >> 4); a < n; a += NT / 16) {
+        } else if ((warp & 3) >= 2 && j >= 0) {
+            for (int a = j + 2 + (ut >> 4); a < n; a += NT / 32) {
                 const double f = A[j * LDS + a];
-                for (int b = a + (tid & 15); b < n; b += 16) A[a * LDS + b] = fma(-f, A[j * LDS + b], A[a * LDS + b]);
+                for (int b = a + (ut & 15); b < n; b += 16) A[a * LDS + b] = fma(-f, A[j * LDS + b], A[a * LDS + b]);
             }
-        } else {
-            for (int l = tid; l < n; l += NT) A[j * LDS + l] = 0.0;
         }
         bsync();
+        if (stop[(j + 1) & 1]) return false;
     }
     return true;
 }
