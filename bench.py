@@ -56,9 +56,9 @@ def _peaks():
 # FP64 rate of GB300 from the profiling recipe's nominal table (1.25 TFLOP/s).
 FP64_PEAK_TFLOPS = 1.25
 
-# ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram launch on the
-# 64^3 case (n = 262,144, m = 64): 446.1 MB, i.e. bytes per (row x trial column);
-# the traffic grows in proportion to n m.
+# ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram launch (the FP64
+# pipe's Gram, B given) on the 64^3 case (n = 262,144, m = 64): 446.1 MB, i.e. bytes
+# per (row x trial column); the traffic grows in proportion to n m.
 GRAM_DRAM_BYTES_PER_ROW_COL = 446.1e6 / (262144 * 64)
 # the same for the double-word Gram k_gram_dw (m = 64 launch on the 64^3
 # case: 402.8 MB read + 3.8 MB written)
@@ -178,7 +178,7 @@ def _fp32_simt_peak_tflops(sm_mhz):
 PHASE_KERNELS = {
     "stencil": "k_lap_axpby / k_lap_shifts (FP64) and k_lap32 (FP32) stencil products",
     "preconditioner": "AV-MG V-cycle kernels (FP64 form; double-word in the mixed form's FP64 phase)",
-    "gram": "k_gram (FP64 multi-Gram; k_gram_dw double-word in the mixed form's FP64 phase)",
+    "gram": "k_gram_fx (tcgen05 multi-Gram on exact fixed-point slices, FP64 accuracy)",
     "update": "k_update (FP64; k_update_dw double-word in the mixed form's FP64 phase)",
     "residual": "k_residual (residual block and column norms)",
     "preconditioner_f32": "FP32 AV-MG V-cycle kernels",
@@ -195,12 +195,13 @@ def _rooflines(prof, peaks, sm_max_mhz, mixed, tensor_cores=True):
     tensor rate as a second figure: the double-word multiply-add costs 13
     FP32 instructions for 2 FP64-equivalent flops (roof = FP32 lane rate / 13),
     the FP64 kernels run at the FP64 rate of the profiling recipe, and the
-    tensor-core Gram executes six BF16 slice products per useful product."""
+    tensor-core Grams execute six (FP32 form) or 22 (FP64 and double-word forms)
+    BF16 products per useful product."""
     out = []
     fp32_peak = _fp32_simt_peak_tflops(sm_max_mhz or 2070.0)
     dw_peak = fp32_peak / 13.0
     alu = {
-        "gram": ("double-word FP32-pipe roof" if mixed else "FP64 rate", dw_peak if mixed else FP64_PEAK_TFLOPS, 1.0),
+        "gram": ("BF16 tensor rate (22 digit products per product)", peaks["bf16_tflops"], 22.0),
         "update": ("double-word FP32-pipe roof" if mixed else "FP64 rate", dw_peak if mixed else FP64_PEAK_TFLOPS,
                    1.0),
         "gram_f32": (("BF16 tensor rate (6 slice products per product)", peaks["bf16_tflops"], 6.0) if tensor_cores

@@ -370,8 +370,8 @@ plhr_status plhr_solve(const plhr_op* A, const plhr_op* B, double sigma, int k,
  * status (device, 3 ints): [0 ok / 1 G_L not positive definite / 2 QR did not
  * converge / 3 rank loss, columns kept, units selected]; clk (device, 16 long
  * long, optional): clock64 stamps of the stages in [0..8] (the stage runs as
- * three launches: [0..2] and [5..8] come from the first and last, [3], [4]
- * bracket the QR iteration in the middle one; SM clocks of different launches
+ * four launches: [0..2] come from the first, [3], [4] bracket the QR iteration
+ * in the second, [5..8] come from the last; SM clocks of different launches
  * are not comparable), the number of QR sweeps in [9] and of bulge-chase
  * steps in [10].  m <= 64, kp <= 16. */
 plhr_status plhr_tharm_extract(int m, int kp, int nv, const double* Gzz, const double* Guq,

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kT) k_restrict_line(Ld gf, Ld gc, int lin, con
 // Linear restriction in 3D, four coarse lines (2 along y x 2 along z) per CTA: a fine
 // value is read 2.25 times instead of 4, six independent loads at a time instead of
 // one after the other.  The weights are 1 and 3, the power of two comes last
-// (96 x 80 x 64 x 16: 69 -> 27 us).
+// (96 x 80 x 64 x 11: 69 -> 27 us).
 constexpr int kQuadT = 512;
 constexpr size_t kQuadSmemMax = 96 * 1024;
 __global__ void __launch_bounds__(kQuadT) k_restrict_quad(Ld gf, Ld gc, const dw* __restrict__ f,

@@ -458,7 +458,8 @@ __device__ __forceinline__ bool francis_eigenvalues(double* Hd, int n, long long
         {
             bool small = t == 0;
             if (t > 0 && t <= hi) {
-                const float s = fmaxf(fabsf(H[(t - 1) * LDS + t - 1].hi) + fabsf(H[t * LDS + t].hi), hnorm);
+                float s = fabsf(H[(t - 1) * LDS + t - 1].hi) + fabsf(H[t * LDS + t].hi);
+                if (s < hnorm) s = hnorm;
                 small = fabsf(H[t * LDS + t - 1].hi) <= eps * s;
             }
             const unsigned b = __ballot_sync(0xffffffffu, small);
