@@ -93,10 +93,14 @@ __global__ void __launch_bounds__(kT) k_scale(Ld g, dw om, const dw* __restrict_
     w[e] = dw_mul(om, r[e]);
 }
 
-// wout = win + om (r - L win) = win + om r - (om / h^2) L' win; omih2 = om / h^2
-template <bool D3>
+// wout = win + om (r - L win) = win + om r - (om / h^2) L' win; omih2 = om / h^2.
+// The cycle's last sweep puts out FP64 (leading dimension ldo) instead of a pass of
+// its own (96 x 80 x 64 x 11: 28 us beside a sweep's 35).
+__device__ __forceinline__ void put(dw* o, dw v) { *o = v; }
+__device__ __forceinline__ void put(double* o, dw v) { *o = dw_to_double_fast(v); }
+template <bool D3, typename To>
 __global__ void __launch_bounds__(kT) k_rich(Ld g, dw om, dw omih2, const dw* __restrict__ win,
-                                             const dw* __restrict__ r, dw* __restrict__ wout) {
+                                             const dw* __restrict__ r, To* __restrict__ wout, int64_t ldo) {
     Pos p;
     if (!pos_of(g, p)) return;
     const int64_t e = p.row * g.nc + p.c;
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kT) k_rich(Ld g, dw om, dw omih2, const dw* __
     dwacc a = dwacc_of(wc);
     dwacc_add_mul(a, om, r[e]);
     dwacc_add_mul(a, dw_neg(omih2), l);
-    wout[e] = dwacc_result(a);
+    put(wout + p.row * ldo + p.c, dwacc_result(a));
 }
 
 // t = L x - sig x
@@ -250,13 +254,35 @@ __global__ void __launch_bounds__(kT) k_prolong_line(Ld gf, Ld gc, int lin, cons
     zi[0] = 0; zw[0] = 1.0f;
     if (D3) nzw = pw(lin, iz, gc.nz, zi, zw);
     const int nc = gf.nc, nu = gc.nx * nc;
-    for (int t = threadIdx.x; t < nu; t += blockDim.x) {
-        const int X = t / nc, c = t - X * nc;
-        dwacc acc = {0.0f, 0.0f};
-        for (int a = 0; a < nzw; ++a)
-            for (int b = 0; b < nyw; ++b)
-                dwacc_add_mul_f(acc, wc[(((int64_t)zi[a] * gc.ny + yi[b]) * gc.nx + X) * nc + c], zw[a] * yw[b]);
-        ush[t] = dwacc_result(acc);
+    if (D3 && lin) {
+        // all four taps, the missing ones with weight 0, so that their loads are in
+        // flight together (44 -> 38 us at 96 x 80 x 64 x 11)
+        const dw* q[4];
+        float w[4];
+        for (int o = 0; o < 4; ++o) {
+            const int a = o >> 1, b = o & 1;
+            const bool in = a < nzw && b < nyw;
+            q[o] = wc + ((int64_t)zi[in ? a : 0] * gc.ny + yi[in ? b : 0]) * nu;
+            w[o] = in ? zw[a] * yw[b] : 0.0f;
+        }
+        for (int t = threadIdx.x; t < nu; t += blockDim.x) {
+            const dw v0 = q[0][t], v1 = q[1][t], v2 = q[2][t], v3 = q[3][t];
+            dwacc acc = {0.0f, 0.0f};
+            dwacc_add_mul_f(acc, v0, w[0]);
+            dwacc_add_mul_f(acc, v1, w[1]);
+            dwacc_add_mul_f(acc, v2, w[2]);
+            dwacc_add_mul_f(acc, v3, w[3]);
+            ush[t] = dwacc_result(acc);
+        }
+    } else {
+        for (int t = threadIdx.x; t < nu; t += blockDim.x) {
+            const int X = t / nc, c = t - X * nc;
+            dwacc acc = {0.0f, 0.0f};
+            for (int a = 0; a < nzw; ++a)
+                for (int b = 0; b < nyw; ++b)
+                    dwacc_add_mul_f(acc, wc[(((int64_t)zi[a] * gc.ny + yi[b]) * gc.nx + X) * nc + c], zw[a] * yw[b]);
+            ush[t] = dwacc_result(acc);
+        }
     }
     __syncthreads();
     const int nf = gf.nx * nc;
@@ -484,20 +510,32 @@ struct Bufs {
         count_launches(1);                                                         \
     } while (0)
 
+template <typename To>
+void rich(const MGLevel& L, int nc, const dw* win, const dw* r, To* wout, int64_t ldo, cudaStream_t s) {
+    auto kern = L.g.d == 3 ? k_rich<true, To> : k_rich<false, To>;
+    kern<<<grid_of(L.g, nc), kT, 0, s>>>(ld_of(L.g, nc), dw_host(L.omega), dw_host(L.omega * L.g.inv_h2()), win, r, wout,
+                                         ldo);
+    count_launches(1);
+}
+
 void sweep(const MGLevel& L, dw sig, int nc, const dw* win, const dw* r, dw* tmp, dw* wout, cudaStream_t s) {
+    if (!L.poly) {
+        rich(L, nc, win, r, wout, nc, s);
+        return;
+    }
     const Ld g = ld_of(L.g, nc);
     const dim3 gr = grid_of(L.g, nc);
     const bool d3 = L.g.d == 3;
-    if (!L.poly) {
-        PLHR_LD(k_rich, gr, g, dw_host(L.omega), dw_host(L.omega * L.g.inv_h2()), win, r, wout);
-        return;
-    }
     PLHR_LD(k_shifted, gr, g, sig, win, tmp);
     PLHR_LD(k_poly, gr, g, sig, dw_host(L.c * L.c), dw_host(0.5 / L.c), dw_host(L.omega), 0, win, tmp, r, wout);
 }
 
+// whether the last sweep of the cycle puts out FP64
+bool sweep_out(const MGHierarchy& H) { return H.lev.size() > 1 && !H.lev.back().poly && H.nu >= 1; }
+
+// out: the result, or out64 (leading dimension ldo) on the finest level where sweep_out
 cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, const std::vector<Bufs>& B,
-                   cudaStream_t s) {
+                   cudaStream_t s, double* out64 = nullptr, int64_t ldo = 0) {
     if (l == 0) {
         const Grid& g0 = H.lev[0].g;
         if (coarse_split<CoarseDw>(g0, nc)) {
@@ -581,6 +619,10 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, co
         PLHR_LD(k_prolong_add, gr, g, gc, H.linear, bf.wc, cur);
     }
     for (int i = 0; i < H.nu; ++i) {
+        if (out64 && i == H.nu - 1) {
+            rich(L, nc, cur, r, out64, ldo, s);
+            break;
+        }
         dw* dst = (i == H.nu - 1) ? out : nxt;
         sweep(L, sig, nc, cur, r, bf.tmp, dst, s);
         nxt = cur;
@@ -624,8 +666,9 @@ cudaError_t mg_vcycle_dw(const MGHierarchy& H, int nc, const double* r, int64_t 
         count_launches(1);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = vcycle(H, top, nc, rdw, wdw, B, st);
-        if (e != cudaSuccess) return e;
+        const bool fused = sweep_out(H);
+        e = vcycle(H, top, nc, rdw, wdw, B, st, fused ? w : nullptr, ldw);
+        if (e != cudaSuccess || fused) return e;
         k_from_dw<<<blocks, 256, 0, st>>>(n, nc, wdw, w, ldw);
         count_launches(1);
         return cudaGetLastError();
