@@ -215,68 +215,84 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(int64_t n, int m, int nb,
 }
 
 // ------------------------------------------------------------------ update
-constexpr int kUpdRows = 32;
-
 // new P = Zraw C_P (m x kp), new V = V C_VV (kp x kp) + new P, for one family,
 // in place: every output row depends only on the same input row, and a chunk
 // is fully staged before any of its rows is written.
-// dotV (optional): the matching block of the new V (already updated); the
-// kernel then accumulates, per column, sum_i out_ij * dotV_ij and
-// sum_i dotV_ij^2 in fixed row order into partial[block][2*kp].
-__global__ void __launch_bounds__(kThreads) k_update(int64_t n, int m, int kp, int nb, FamPtrs F,
+//
+// The FP64 pipe binds (m + kp multiply-adds per output), if it is kept fed: thread
+// t owns column j = t % kp of rows r = t / kp and r + `rows` of a chunk of 2 rows
+// rows, `rows` as large as the threads allow, so that no warp idles whatever kp is,
+// and the next chunk's values are on their way in registers meanwhile
+// (both families of a 48^3 Hamiltonian's iteration, k' = 12: 180 -> 147 us).
+__global__ void __launch_bounds__(kThreads) k_update(int64_t n, int m, int kp, int nb, int rows, FamPtrs F,
                                                      const double* __restrict__ Cp,
                                                      const double* __restrict__ Cvv,
                                                      double* __restrict__ Vout, int64_t ldvo,
-                                                     double* __restrict__ Pout, int64_t ldpo,
-                                                     const double* __restrict__ dotV, int64_t lddv,
-                                                     double* __restrict__ partial) {
+                                                     double* __restrict__ Pout, int64_t ldpo) {
     extern __shared__ double sh[];
     double* sc = sh;                        // C_P [m][kp]
     double* sv = sc + m * kp;               // C_VV [kp][kp]
-    double* srow = sv + kp * kp;            // [kUpdRows][m]
-    double* sout = srow + kUpdRows * m;     // [kUpdRows][kp] new V-part values
-    double* sd = sout + kUpdRows * kp;      // [kUpdRows][kp] dotV values
-    for (int t = threadIdx.x; t < m * kp; t += blockDim.x) sc[t] = Cp[t];
-    for (int t = threadIdx.x; t < kp * kp; t += blockDim.x) sv[t] = Cvv[t];
-    double acc_a = 0.0, acc_b = 0.0;        // owned by threads j < kp
-    const int64_t nchunks = (n + kUpdRows - 1) / kUpdRows;
-    __syncthreads();
+    double* srow = sv + kp * kp;            // [2 rows][m]
+    const int tid = threadIdx.x;
+    for (int t = tid; t < m * kp; t += kThreads) sc[t] = Cp[t];
+    for (int t = tid; t < kp * kp; t += kThreads) sv[t] = Cvv[t];
+    const int chunk = 2 * rows, r0 = tid / kp, j = tid - r0 * kp;
+    const int64_t nchunks = (n + chunk - 1) / chunk;
+    double next[4][2];
+    auto fetch = [&](int64_t ch) {
+        const int64_t row0 = ch * chunk;
+        const int nrows = (int)((n - row0) < chunk ? (n - row0) : chunk);
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int t = tid + k * kThreads;
+                if (b < nb && t < nrows * F.nc[b]) {
+                    const int r = t / F.nc[b], c = t - r * F.nc[b];
+                    next[b][k] = F.p[b][(row0 + r) * F.ld[b] + c];
+                }
+            }
+    };
+    if (blockIdx.x < nchunks) fetch(blockIdx.x);
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        int64_t row0 = ch * kUpdRows;
-        int nrows = (int)((n - row0) < kUpdRows ? (n - row0) : kUpdRows);
-        stage_rows(srow, m, row0, nrows, F, nb);
-        if (dotV)
-            for (int t = threadIdx.x; t < nrows * kp; t += blockDim.x) {
-                int r = t / kp, j = t - r * kp;
-                sd[t] = dotV[(row0 + r) * lddv + j];
+        const int64_t row0 = ch * chunk;
+        const int nrows = (int)((n - row0) < chunk ? (n - row0) : chunk);
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int t = tid + k * kThreads;
+                if (b < nb && t < nrows * F.nc[b]) {
+                    const int r = t / F.nc[b], c = t - r * F.nc[b];
+                    srow[r * m + F.off[b] + c] = next[b][k];
+                }
             }
         __syncthreads();
-        for (int t = threadIdx.x; t < nrows * kp; t += blockDim.x) {
-            int r = t / kp, j = t - r * kp;
-            const double* z = srow + r * m;
-            double p = 0.0;
-            for (int i = 0; i < m; ++i) p = fma(z[i], sc[i * kp + j], p);
-            double v = p;
-            for (int i = 0; i < kp; ++i) v = fma(z[i], sv[i * kp + j], v);
-            int64_t row = row0 + r;
-            Pout[row * ldpo + j] = p;
-            Vout[row * ldvo + j] = v;
-            sout[t] = v;
+        if (ch + gridDim.x < nchunks) fetch(ch + gridDim.x);
+        if (r0 >= rows || r0 >= nrows) continue;
+        const bool two = r0 + rows < nrows;
+        const double* z0 = srow + r0 * m;
+        const double* z1 = srow + (two ? r0 + rows : r0) * m;
+        double p0 = 0.0, p1 = 0.0;
+        for (int i = 0; i < m; ++i) {
+            const double c = sc[i * kp + j];
+            p0 = fma(z0[i], c, p0);
+            p1 = fma(z1[i], c, p1);
         }
-        __syncthreads();
-        if (dotV && threadIdx.x < kp) {
-            int j = threadIdx.x;
-            for (int r = 0; r < nrows; ++r) {
-                double d = sd[r * kp + j];
-                acc_a = fma(sout[r * kp + j], d, acc_a);
-                acc_b = fma(d, d, acc_b);
-            }
+        double v0 = p0, v1 = p1;
+        for (int i = 0; i < kp; ++i) {
+            const double c = sv[i * kp + j];
+            v0 = fma(z0[i], c, v0);
+            v1 = fma(z1[i], c, v1);
         }
-        __syncthreads();
-    }
-    if (dotV && threadIdx.x < kp) {
-        partial[(int64_t)blockIdx.x * 2 * kp + threadIdx.x] = acc_a;
-        partial[(int64_t)blockIdx.x * 2 * kp + kp + threadIdx.x] = acc_b;
+        const int64_t row = row0 + r0;
+        Pout[row * ldpo + j] = p0;
+        Vout[row * ldvo + j] = v0;
+        if (two) {
+            Pout[(row + rows) * ldpo + j] = p1;
+            Vout[(row + rows) * ldvo + j] = v1;
+        }
     }
 }
 
@@ -353,24 +369,22 @@ int gram_max_m() {
 }
 
 cudaError_t block_update(int64_t n, int nb, const Blk<const double>* F, int kp, const double* Cp,
-                         const double* Cvv, double* Vout, int64_t ldvo, double* Pout, int64_t ldpo,
-                         const double* dotV, int64_t lddv, double* partial, double* out, cudaStream_t s) {
+                         const double* Cvv, double* Vout, int64_t ldvo, double* Pout, int64_t ldpo, cudaStream_t s) {
     FamPtrs FF = fam_of(F, nb);
-    int m = 0;
-    for (int i = 0; i < nb; ++i) m += F[i].nc;
-    int blocks = reduce_blocks();
-    size_t shm = sizeof(double) * (m * kp + kp * kp + kUpdRows * m + 2 * kUpdRows * kp);
-    k_update<<<blocks, kThreads, shm, s>>>(n, m, kp, nb, FF, Cp, Cvv, Vout, ldvo, Pout, ldpo, dotV, lddv,
-                                           partial);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (dotV) {
-        k_sum_partials<<<sum_grid(2 * kp), 256, 0, s>>>(blocks, 2 * kp, partial, out);
-        count_launches(1);
-        e = cudaGetLastError();
+    int m = 0, widest = kp;
+    for (int i = 0; i < nb; ++i) {
+        m += F[i].nc;
+        widest = F[i].nc > widest ? F[i].nc : widest;
     }
-    return e;
+    if (widest > kThreads) return cudaErrorInvalidValue;
+    const int rows = kThreads / widest;   // a family's values of a chunk: at most two per thread
+    const size_t shm = sizeof(double) * (m * kp + kp * kp + 2 * rows * m);
+    const cudaError_t e = shm > 48 * 1024
+        ? cudaFuncSetAttribute(k_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    k_update<<<sm_count() * 3, kThreads, shm, s>>>(n, m, kp, nb, rows, FF, Cp, Cvv, Vout, ldvo, Pout, ldpo);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 }  // namespace plhr

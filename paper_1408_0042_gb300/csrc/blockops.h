@@ -90,11 +90,9 @@ cudaError_t shift_combine(int64_t n, int nc, const double* AX, int64_t ldax, con
                           cudaStream_t s);
 
 // Family F = [F_0 .. F_{nb-1}] (m columns): Pout = F C_P, Vout = F_0 C_VV + F C_P
-// (in place allowed: Vout may be F_0, Pout may be F_{nb-1}).  When dotV is
-// given, out[0:kp] = sum Vout .* dotV, out[kp:2kp] = sum dotV .^ 2.
+// (in place allowed: Vout may be F_0, Pout may be F_{nb-1}).
 cudaError_t block_update(int64_t n, int nb, const Blk<const double>* F, int kp, const double* Cp,
-                         const double* Cvv, double* Vout, int64_t ldvo, double* Pout, int64_t ldpo,
-                         const double* dotV, int64_t lddv, double* partial, double* out, cudaStream_t s);
+                         const double* Cvv, double* Vout, int64_t ldvo, double* Pout, int64_t ldpo, cudaStream_t s);
 
 // Y = X C for X n x kx (ldx), C kx x ky (row-major); in place allowed when
 // ky <= kx and Y == X (rows are staged).

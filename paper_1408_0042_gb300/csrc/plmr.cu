@@ -317,7 +317,7 @@ plhr_status plmr_solve(const plhr_op* A, const plhr_op* B, plhr_prec* T, double 
         {
             PhaseScope ps(PH_UPDATE, s, 2.0 * n * nb, 8.0 * n * (nb + 2));
             // p = Z Cp (the v entry of Cp is zero), v = v Cvv + p
-            PLHR_TRY_CUDA(block_update(n, nb, zb, 1, Cp, Cvv, vec[V], 1, vec[P], 1, nullptr, 0, nullptr, nullptr, s));
+            PLHR_TRY_CUDA(block_update(n, nb, zb, 1, Cp, Cvv, vec[V], 1, vec[P], 1, s));
         }
         have_p = true;
         PLHR_TRY(prod(vec[V], vec[AV], vec[BV], nullptr));
