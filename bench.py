@@ -56,13 +56,10 @@ def _peaks():
 # FP64 rate of GB300 from the profiling recipe's nominal table (1.25 TFLOP/s).
 FP64_PEAK_TFLOPS = 1.25
 
-# ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram launch (the FP64
-# pipe's Gram, B given) on the 64^3 case (n = 262,144, m = 64): 446.1 MB, i.e. bytes
-# per (row x trial column); the traffic grows in proportion to n m.
-GRAM_DRAM_BYTES_PER_ROW_COL = 446.1e6 / (262144 * 64)
-# the same for the double-word Gram k_gram_dw (m = 64 launch on the 64^3
-# case: 402.8 MB read + 3.8 MB written)
-GRAM_DW_DRAM_BYTES_PER_ROW_COL = 406.60e6 / (262144 * 64)
+# ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram_fx launch
+# (n = 262,144, m = 36: the three blocks once, 226.5 MB), i.e. bytes per (row x trial column); the traffic
+# grows in proportion to n m.
+GRAM_DRAM_BYTES_PER_ROW_COL = 226.5e6 / (262144 * 36)
 
 
 class ClockSampler:
@@ -350,12 +347,11 @@ def run_ours(args, world, rank, local):
         if dom["phase"] == "gram":
             # ncu DRAM bytes per (row x trial column) of the kernel, scaled to the
             # average launch of this run (the algorithmic bytes are 3 n m x 8)
-            per = GRAM_DRAM_BYTES_PER_ROW_COL if args.precision == "f64" else GRAM_DW_DRAM_BYTES_PER_ROW_COL
+            per = GRAM_DRAM_BYTES_PER_ROW_COL
             m_avg = dom["bytes_per_call"] / (24.0 * n)
             dom["traffic"] = per * n * m_avg
-            dom["traffic_note"] = ("ncu dram__bytes_read + write of one %s launch with m = 64 on the 64^3 case, "
-                                   "scaled by n m to this run's average launch (n = %d, m = %.1f)" % (
-                                       "k_gram" if args.precision == "f64" else "k_gram_dw", n, m_avg))
+            dom["traffic_note"] = ("ncu dram__bytes_read + write of one k_gram_fx launch (n = 262,144, m = 36), "
+                                   "scaled by n m to this run's average launch (n = %d, m = %.1f)" % (n, m_avg))
     dense = prof.get("dense", {})
     dense_stage = {"ms_per_iteration": dense["ms"] / dense["calls"] if dense.get("calls") else None,
                    "ms_per_step": dense.get("ms", 0.0) / max(1, args.steps),

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(int64_t n, int m, int nb,
 // t owns column j = t % kp of rows r = t / kp and r + `rows` of a chunk of 2 rows
 // rows, `rows` as large as the threads allow, so that no warp idles whatever kp is,
 // and the next chunk's values are on their way in registers meanwhile
-// (both families of a 48^3 Hamiltonian's iteration, k' = 12: 180 -> 147 us).
+// (both families of a 48^3 Hamiltonian's iteration: 180 -> 147 us).
 __global__ void __launch_bounds__(kThreads) k_update(int64_t n, int m, int kp, int nb, int rows, FamPtrs F,
                                                      const double* __restrict__ Cp,
                                                      const double* __restrict__ Cvv,

@@ -1,5 +1,4 @@
-// Small dense FP64 stage of one PLHR iteration, run by a single warp on the
-// device (no host round trip).  Input: the raw Grams of the trial basis
+// Small dense stage of one PLHR iteration on the device (no host round trip).  Input: the raw Grams of the trial basis
 // Z = [V W S P] (Z*Z, U*Q with U = AZ - sigma Z, Q*Z, Q = T U) and the column
 // scales of Z.  Steps:
 //  1. B-orthonormalisation of Z (Alg. 2 step 6) done implicitly: with the
@@ -12,9 +11,9 @@
 //     (Eq. THarm_evp_sinv): G_L = L L^T, C = L^-1 G_R L^-T, eigenpairs (tau, z)
 //     of C, y = L^-T z.
 //  3. Eigenvalues of C: Householder reduction to Hessenberg form and the
-//     Francis double-shift QR iteration with Schur vectors (Golub & Van Loan,
-//     "Matrix Computations", Sec. 7.4-7.5); eigenvectors of the quasi-triangular
-//     Schur factor by back substitution.
+//     Francis double-shift QR iteration, eigenvalues only (Golub & Van Loan,
+//     "Matrix Computations", Sec. 7.4-7.5); eigenvectors of the selected ones by
+//     inverse iteration on the Hessenberg form.
 //  4. Order by |xi| with each complex xi followed by its conjugate, select k'
 //     (Alg. 3 steps 7-10), rotate complex y so Re(y) is orthogonal to Im(y)
 //     and the longer of the two, build the real Y' = [Y0 YR yR~ YI].
@@ -296,7 +295,7 @@ __device__ void bhessenberg(double* Hd, double* Vhd, double* betad, int n, doubl
     bsync();
 }
 
-// ---------------------------------------------------------------- eigenvalues (one warp)
+// ---------------------------------------------------------------- eigenvalues (three warps)
 // Householder vector for (x, y, z) in double-word arithmetic: u = (1, u1, u2),
 // tau and beta with (I - tau u u^T)(x, y, z)^T = (beta, 0, 0)^T.
 //
