@@ -57,9 +57,9 @@ def _peaks():
 FP64_PEAK_TFLOPS = 1.25
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram_fx launch
-# (n = 262,144, m = 36: the three blocks once, 226.5 MB), i.e. bytes per (row x trial column); the traffic
+# (n = 262,144, m = 36: 231.9 MB read, 6.0 MB written), i.e. bytes per (row x trial column); the traffic
 # grows in proportion to n m.
-GRAM_DRAM_BYTES_PER_ROW_COL = 226.5e6 / (262144 * 36)
+GRAM_DRAM_BYTES_PER_ROW_COL = 237.9e6 / (262144 * 36)
 
 
 class ClockSampler:
