@@ -40,9 +40,11 @@ FamD fam_d(const Blk<const double>* b, int nb) {
 // row and a chunk is staged before any of its rows is written)
 // Thread t owns column j = t % kp of rows r = t / kp and r + `rows` of each chunk
 // of 2 `rows` rows: the two rows share the coefficient loads and give each thread two
-// independent sums.  The next chunk's values are on their way in registers
-// meanwhile.  Every output is summed over i in the same order as with one output
-// per thread (both families of an iteration at 112 x 96 x 80: 788 -> 720 us).
+// independent sums.  Every output is summed over i in the same order as with one
+// output per thread.  A chunk has as many rows as the threads allow, so that no warp
+// idles where k' does not divide 256 (both families of an iteration at
+// 112 x 96 x 80: 788 -> 692 us; fetching the next chunk into registers meanwhile
+// was 4 % slower at 128^3, k' = 16).
 __global__ void __launch_bounds__(256) k_update_dw(int64_t n, int m, int kp, int nb, int rows, FamD F,
                                                    const double* __restrict__ Cp, const double* __restrict__ Cvv,
                                                    double* __restrict__ Vout, int64_t ldvo, double* __restrict__ Pout,
@@ -50,43 +52,25 @@ __global__ void __launch_bounds__(256) k_update_dw(int64_t n, int m, int kp, int
     extern __shared__ __align__(16) unsigned char raw[];
     dw* cp = reinterpret_cast<dw*>(raw);      // [m][kp]
     dw* cv = cp + m * kp;                     // [kp][kp]
-    dw* zr = cv + kp * kp;                    // [rows][m]
+    dw* zr = cv + kp * kp;                    // [2 rows][m]
     for (int t = threadIdx.x; t < m * kp; t += blockDim.x) cp[t] = dw_from_double(Cp[t]);
     for (int t = threadIdx.x; t < kp * kp; t += blockDim.x) cv[t] = dw_from_double(Cvv[t]);
     const int tid = threadIdx.x, chunk = 2 * rows, r0 = tid / kp, j = tid - r0 * kp;
     const int64_t nchunks = (n + chunk - 1) / chunk;
-    double next[4][2];
-    auto fetch = [&](int64_t ch) {
-        const int64_t row0 = ch * chunk;
-        const int nrows = (int)((n - row0) < chunk ? (n - row0) : chunk);
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int t = tid + k * 256;
-                if (b < nb && t < nrows * F.nc[b]) {
-                    const int r = t / F.nc[b], c = t - r * F.nc[b];
-                    next[b][k] = F.p[b][(row0 + r) * F.ld[b] + c];
-                }
-            }
-    };
-    if (blockIdx.x < nchunks) fetch(blockIdx.x);
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
         const int64_t row0 = ch * chunk;
         const int nrows = (int)((n - row0) < chunk ? (n - row0) : chunk);
         __syncthreads();
 #pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int t = tid + k * 256;
-                if (b < nb && t < nrows * F.nc[b]) {
-                    const int r = t / F.nc[b], c = t - r * F.nc[b];
-                    zr[r * m + F.off[b] + c] = dw_split_trunc(next[b][k]);
-                }
+        for (int b = 0; b < 4; ++b) {
+            if (b >= nb) break;
+            const int nc = F.nc[b];
+            for (int t = tid; t < nrows * nc; t += 256) {
+                const int r = t / nc, c = t - r * nc;
+                zr[r * m + F.off[b] + c] = dw_split_trunc(F.p[b][(row0 + r) * F.ld[b] + c]);
             }
+        }
         __syncthreads();
-        if (ch + gridDim.x < nchunks) fetch(ch + gridDim.x);
         if (r0 >= rows || r0 >= nrows) continue;
         const bool two = r0 + rows < nrows;
         const dw* z0 = zr + r0 * m;
