@@ -1406,8 +1406,27 @@ __global__ void k_rq(int kp, const double* dots, const int* tags, const int* par
     }
 }
 
+// columns in order by |th - sigma| (ties: smaller th first), one thread
+__device__ void rr_order(const double* th, int n, double sigma, int* ord) {
+    for (int j = 0; j < n; ++j) ord[j] = j;
+    for (int i = 1; i < n; ++i) {
+        int o = ord[i];
+        double d = fabs(th[o] - sigma), l = th[o];
+        int j = i - 1;
+        while (j >= 0) {
+            int p = ord[j];
+            double dp = fabs(th[p] - sigma);
+            if (dp > d || (dp == d && th[p] > l)) { ord[j + 1] = p; --j; }
+            else break;
+        }
+        ord[j + 1] = o;
+    }
+}
+
 // one warp: Cholesky of GB, M = L^-1 GA L^-T, cyclic Jacobi (Golub & Van Loan
-// Sec. 8.5), C = L^-T W, sort by |theta - sigma|.
+// Sec. 8.5), C = L^-T W, sort by |theta - sigma|.  Where GB has no Cholesky factor
+// (ok_out 0) the columns are only scaled and sorted, theta their Rayleigh
+// quotients: a block that is multiplied by C all the same keeps its columns.
 __global__ void __launch_bounds__(32) k_rr(int n, const double* GA, const double* GB, double sigma,
                                            const double* rowscale, double* C, double* theta, int* ok_out) {
     __shared__ double L[32 * 33], M[32 * 33], W[32 * 33];
@@ -1422,7 +1441,18 @@ __global__ void __launch_bounds__(32) k_rr(int n, const double* GA, const double
     }
     __syncwarp();
     if (!chol_lower(L, n, ld)) {
-        if (lane == 0) *ok_out = 0;
+        if (lane < n) th[lane] = GA[lane * n + lane] / GB[lane * n + lane];
+        __syncwarp();
+        if (lane == 0) {
+            rr_order(th, n, sigma, ord);
+            *ok_out = 0;
+        }
+        __syncwarp();
+        for (int i = lane; i < n * n; i += 32) {
+            const int r = i / n, c = i % n;
+            C[i] = r == ord[c] ? (rowscale ? rowscale[r] : 1.0) : 0.0;
+        }
+        if (lane < n) theta[lane] = th[ord[lane]];
         return;
     }
     // M <- L^-1 M L^-T
@@ -1487,19 +1517,8 @@ __global__ void __launch_bounds__(32) k_rr(int n, const double* GA, const double
             }
     }
     if (lane == 0) {
-        for (int j = 0; j < n; ++j) { th[j] = M[j * ld + j]; ord[j] = j; }
-        for (int i = 1; i < n; ++i) {
-            int o = ord[i];
-            double d = fabs(th[o] - sigma), l = th[o];
-            int j = i - 1;
-            while (j >= 0) {
-                int p = ord[j];
-                double dp = fabs(th[p] - sigma);
-                if (dp > d || (dp == d && th[p] > l)) { ord[j + 1] = p; --j; }
-                else break;
-            }
-            ord[j + 1] = o;
-        }
+        for (int j = 0; j < n; ++j) th[j] = M[j * ld + j];
+        rr_order(th, n, sigma, ord);
     }
     __syncwarp();
     // C = L^-T W (back substitution per column), columns reordered

@@ -54,7 +54,8 @@ cudaError_t dense_rq(int kp, const double* dots, const int* tags, const int* par
 // Standard Rayleigh-Ritz (Alg. 2 step 12): G_A c = theta G_B c for kp x kp
 // Grams; C (kp x kp, columns ordered by |theta - sigma|, ties by theta) and theta.
 // rowscale (kp, optional): C rows are multiplied by it (Ritz coefficients on
-// the stored, unscaled columns).
+// the stored, unscaled columns).  ok 0 where G_B has no Cholesky factor: C then only
+// scales and sorts the columns, theta are their Rayleigh quotients.
 cudaError_t dense_rr(int kp, const double* GA, const double* GB, double sigma, const double* rowscale, double* C,
                      double* theta, int* ok, cudaStream_t s);
 
