@@ -421,9 +421,14 @@ plhr_status plhr_tharm_extract_noalloc(int m, int kp, int nv, const double* Gzz,
  * has n rows, element (i, j) at Z[b][i * ldz[b] + j] (host arrays of device
  * pointers and leading dimensions).  Forms:
  *   PLHR_GRAM_F64     FP64 blocks, FP64-class products and sums: six 9-bit
- *                     slices per value and exact integer sums on the tensor
- *                     cores, errors about 2^-51 |x| |y| (FP64 multiply-adds
- *                     when a column holds Inf or NaN);
+ *                     slices per value and integer sums on the tensor cores.
+ *                     Errors are relative to the columns' norms, not to the
+ *                     entry: about 2^-51 |x| |y| (2^-43 at most) where a
+ *                     column's entries are of one size; columns with few large
+ *                     entries and a long tail of equal low digits lose up to
+ *                     2^-40 of the product of their largest entries for every
+ *                     128 rows that an SM takes (of n / SMs).  FP64
+ *                     multiply-adds when a column holds Inf or NaN;
  *   PLHR_GRAM_F32     FP32 blocks, FP32 products on the FP32 pipes, sums
  *                     folded into double-FP32 every 32 rows;
  *   PLHR_GRAM_DW      FP64 blocks, the form of the mixed solve's FP64-storage

@@ -17,24 +17,32 @@
 // of base 2^9, d_k in [-256, 256], k = 0 the leading one.  Every such digit is
 // a BF16 number (8 significant bits and a sign), also when it is stored as
 // d_k 2^-9k.  The product of digits k and l of two values belongs to level
-// k + l; levels 0 to 5 (21 products) and the square of digit 3, which alone of
-// level 6 is not of random sign on the diagonal, are formed.  The rest is below
-// 2^-51 of the product of the two column magnitudes and averages out.
+// k + l; levels 0 to 6 (26 products) are formed, of U^T Q level 7 too, which its
+// MMAs of two levels bring with them.  The rest is below 2^-63 of 2^E 2^E' a row.
 // Sums: over a period of 128 rows a level of L + 1 products is at most
-// (L + 1) 128 2^16, so levels 0 and 1 always, and levels 2 and 3 except for
-// columns of nearly constant magnitude, accumulate exactly in FP32 tensor
-// memory.  Levels 4 and 5 are 2^-36 of the leading one and may round.  At the
+// (L + 1) 128 2^16 (its two products with a leading digit, which is below 2^7, half
+// of that), so levels 0 to 2, and level 3 except where all its products are near
+// their largest, accumulate exactly in FP32 tensor memory.  Levels 4 to 6 share an
+// accumulator, which drops what is below 2^-24 of its content with each MMA.  At the
 // end of a period the accumulators are read back as integers into 64-bit sums
-// in units of 2^-34 of the leading digit product.  Measured on the trial bases of a Laplacian
-// (12^3 to 100 x 90 x 80 points, m = 12 to 64) against extended-precision
-// references: largest error over |x| |y| 1.8e-16 to 6e-16, where FP64
-// multiply-adds give 5.7e-16 to 1.5e-15 and double-word ones 5e-15 to 5e-13.
+// in units of 2^-36 of the leading digit product (2^-54 of 2^E 2^E').
+//
+// Accuracy.  On columns whose entries are of one size, such as trial bases, an entry is
+// correct to a few 2^-53 of the column norms: 2e-16 to 9e-16 of |x| |y| at 40,000 to
+// 2,097,152 rows (FP64 multiply-adds 2e-16 to 1.3e-15, double-word ones 5e-15 to
+// 2e-11).  A column with few large entries and a long tail of equal low digits loses
+// up to 2^-40 of the product of the largest entries per 128 rows of an SM (128 MMAs
+// at one unit of the shared accumulator); measured with one entry 1 and 10^-3 to
+// 10^-6 elsewhere at 2,097,152 rows: 1e-13, 2.4e-12 (10^-4), 9e-14 where FP64
+// multiply-adds lose 1e-13, 6e-13, 6e-13.  Without level 6, which has 2 d_1 d_5 and
+// 2 d_2 d_4 of one sign there, it was 1.7e-12, 6.5e-12, 5e-13.
 //
 // Exponents.  E is kept per column and CTA: the largest exponent met so far
-// plus one (plus two in long runs), from 32 rows spread over the CTA's share on.
+// plus two, in long runs from 32 rows spread over the CTA's share on.
 // When a value exceeds it, the pending period is folded, the integers are
-// shifted to the new exponents and the CTA goes on.  So the precision is relative to the columns' norms (what the
-// Cholesky factorisation of a Gram matrix needs), not to each pair of entries.
+// shifted to the new exponents and the CTA goes on.  So the precision is relative to
+// the columns' norms (what the Cholesky factorisation of a Gram matrix needs), not to
+// each pair of entries.
 // A column holding Inf or NaN and a wait that times out set the CTA's flag: the
 // plain FP64 kernel, which is launched behind this one and returns at once
 // otherwise, then redoes the Grams.
@@ -44,8 +52,8 @@
 // Q^T Z; five accumulators hold levels 0, 1, 2, 3 and the rest.  U^T Q fills the
 // 128 lanes with two levels at once: [U_k-1; U_k] with Q_l adds to level
 // k + l - 1 in the upper and k + l in the lower half, so three accumulators hold
-// all six levels and the eight fill the 512 columns of tensor memory at
-// m = 64.  The 70 MMAs of a step take 3.4k cycles (49 each: operand reads from
+// all eight levels and the eight fill the 512 columns of tensor memory at
+// m = 64.  The 86 MMAs of a step take 4.2k cycles (49 each: operand reads from
 // shared memory bind at N = 64).
 //
 // Roles.  Four warps issue the MMAs (issued by a converting warp, that warp
@@ -70,13 +78,14 @@ constexpr int kFxThreads = kFxConv + 128;      // and a warpgroup that issues th
 constexpr int kFxK = 32;                       // rows per step
 constexpr int kMaxPeriod = 4;                  // steps per period
 constexpr int kDigits = 6;
+constexpr int kUnit = 36;                      // the 64-bit sums are in units of 2^-kUnit of the leading digit product
 constexpr int kCore = 128;                     // core matrix: 8 rows x 16 bytes
-// A step's panel: the U digits behind a block of zeros (per core column of 8
-// rows of the step: [0 | U0 | .. | U5], 7 mp operand rows), then per digit a
+// A step's panel: the U digits between two blocks of zeros (per core column of 8
+// rows of the step: [0 | U0 | .. | U5 | 0], 8 mp operand rows), then per digit a
 // slice [Z | Q] of 2 mp operand rows.  Core columns are 64 bytes further apart
 // than their rows take, so that the stores of a warp (4 columns of all 4 core
 // columns) use different banks.
-__host__ __device__ constexpr int lbo_u_of(int mp) { return 7 * 16 * mp + 64; }
+__host__ __device__ constexpr int lbo_u_of(int mp) { return 8 * 16 * mp + 64; }
 __host__ __device__ constexpr int lbo_z_of(int mp) { return 2 * 16 * mp + 64; }
 __host__ __device__ constexpr int panel_of(int mp) { return 4 * (lbo_u_of(mp) + kDigits * lbo_z_of(mp)); }
 constexpr int kFxOperand = 2 * panel_of(64) + 4096;  // A reads 128 rows: up to 2 KB past a narrow last slice
@@ -274,7 +283,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     tc::mma_bf16(d, ad + kz, bd + kz, idesc, 1u);
                 };
                 auto mma_u = [&](uint32_t d, int b, int l, uint32_t accum) {
-                    // [U_b-1; U_b] (U_-1 = 0) with Q_l
+                    // [U_b-1; U_b] (U_-1 = U_6 = 0) with Q_l
                     const uint64_t ad = hu + b * db, bd = hz + l * ds + db;
                     tc::mma_bf16(d, ad, bd, idesc, accum);
                     tc::mma_bf16(d, ad + ku, bd + kz, idesc, 1u);
@@ -289,13 +298,13 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                         mma_u(tmem + (uint32_t)((5 + p) * mp), 2 * p + 1 - l, l, l ? 1u : start);
                 };
                 // every accumulator has one issuer, so the order of its sums is fixed
-                if (share == 0) {            // levels 5 and 4 behind the square of digit 3: the finest first
-                    mma_z(tmem + 4 * mp, 3, 3, carry);
+                if (share == 0) {            // levels 6 to 4, the finest first
+                    for (int k = 1; k <= 5; ++k) mma_z(tmem + 4 * mp, k, 6 - k, k == 1 ? carry : 1u);
                     levels_z(5, 4, 1u);
                 } else if (share == 1) {
                     levels_z(3, 0, carry);
-                } else if (share == 2) {     // levels 4 and 5, the square of digit 3 first
-                    mma_u(tmem + 7 * mp, 4, 3, carry);
+                } else if (share == 2) {     // levels 6 and 7 (U_6 = 0), then 4 and 5
+                    for (int l = 5; l >= 1; --l) mma_u(tmem + 7 * mp, 7 - l, l, l == 5 ? carry : 1u);
                     levels_u(2, 1u);
                 } else {
                     levels_u(1, carry);
@@ -320,6 +329,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
         const int r = 32 * q + lane;
         const bool reads = 32 * q < 2 * mp;
         const float odd = r < mp ? 1.0f : 0x1p9f;          // rows mp.. of the U accumulators hold the odd levels
+        constexpr float fine = (float)(1ull << kUnit);
         unsigned long long az[16], au[16];
 #pragma unroll
         for (int c = 0; c < 16; ++c) { az[c] = 0; au[c] = 0; }
@@ -362,25 +372,26 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                             tc::tmem_ld_wait();
                         };
                         get(0);
-                        add8<34>(az + c, v, 1.0f);
+                        add8<kUnit>(az + c, v, 1.0f);
                         get(1);
-                        add8<25>(az + c, v, 0x1p9f);
+                        add8<kUnit - 9>(az + c, v, 0x1p9f);
                         get(2);
-                        add8<16>(az + c, v, 0x1p18f);
+                        add8<kUnit - 18>(az + c, v, 0x1p18f);
                         get(3);
-                        add8<7>(az + c, v, 0x1p27f);
+                        add8<kUnit - 27>(az + c, v, 0x1p27f);
                         get(4);
-                        add8<0>(az + c, v, 0x1p34f);
+                        add8<0>(az + c, v, fine);
                         get(5);
-                        add8<34>(au + c, v, odd);
+                        add8<kUnit>(au + c, v, odd);
                         get(6);
-                        add8<16>(au + c, v, odd * 0x1p18f);
+                        add8<kUnit - 18>(au + c, v, odd * 0x1p18f);
                         get(7);
-                        add8<0>(au + c, v, odd * 0x1p34f);
+                        add8<0>(au + c, v, odd * fine);
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            az[c + i] -= (kB << 34) + (kB << 25) + (kB << 16) + (kB << 7) + kB;
-                            au[c + i] -= (kB << 34) + (kB << 16) + kB;
+                            az[c + i] -= (kB << kUnit) + (kB << (kUnit - 9)) + (kB << (kUnit - 18)) +
+                                         (kB << (kUnit - 27)) + kB;
+                            au[c + i] -= (kB << kUnit) + (kB << (kUnit - 18)) + kB;
                             const int hz = (int)(az[c + i] >> 32), hu = (int)(au[c + i] >> 32);
                             top |= (unsigned)(hz ^ (hz >> 31)) | (unsigned)(hu ^ (hu >> 31));
                         }
@@ -411,12 +422,13 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     const int i = t >> 5, cc = t & 31;
                     const int y = (cc >> 3) * ncol + c + (cc & 7);
                     if (y >= m || c + (cc & 7) >= ncol) continue;
-                    // units of 2^-34 of a leading digit product; a column's leading digit is
+                    // units of 2^-kUnit of a leading digit product; a column's leading digit is
                     // in units of 2^-9 2^(exponent - 1022)
+                    constexpr double unit = 1.0 / (double)(1ull << (18 + kUnit));
                     if (u) {
                         // even levels in row i, odd ones in row mp + i; the upper triangle, mirrored
                         if (i >= m || i > y) continue;
-                        const double v = (D[i * kLdD + cc] + D[(mp + i) * kLdD + cc] * 0x1p-9) * 0x1p-52 *
+                        const double v = (D[i * kLdD + cc] + D[(mp + i) * kLdD + cc] * 0x1p-9) * unit *
                                          (S.fac[2 * mp + i] * S.fac[mp + y]);
                         double* o = out + m * m;
                         const double s = first ? v : o[i * m + y] + v;
@@ -425,7 +437,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     } else {
                         const int x = i < mp ? i : i - mp;
                         if (i >= 2 * mp || x >= m) continue;
-                        const double v = D[i * kLdD + cc] * 0x1p-52 * (S.fac[i] * S.fac[y]);
+                        const double v = D[i * kLdD + cc] * unit * (S.fac[i] * S.fac[y]);
                         double* o = out + (i < mp ? 0 : 2 * m * m) + x * m + y;
                         *o = first ? v : *o + v;
                     }
@@ -440,8 +452,10 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
             }
         };
 
-        // in a long run, one binade of room: a column then settles after a few steps
-        const int room = nst > 16 ? 2 : 1;
+        // one binade of room: a column then settles after a few steps (32,768 rows, m = 36:
+        // 183 -> 145 us a call), and the leading digit of one whose magnitude hardly changes
+        // stays below 2^7, without which level 2 passes 2^24 and loses up to 1.4e-12 |x| |y|
+        constexpr int room = 2;
         int ez = kExpFloor, eu = kExpFloor, eq = kExpFloor;   // exponents of the thread's column
         int mz = 0, mu = 0, mq = 0;                           // largest exponent fields of the loaded values
         // U = AZ - sigma Z and the exponents of the loaded step
