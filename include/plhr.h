@@ -428,7 +428,9 @@ plhr_status plhr_tharm_extract_noalloc(int m, int kp, int nv, const double* Gzz,
  *                     entries and a long tail of equal low digits lose up to
  *                     2^-40 of the product of their largest entries for every
  *                     128 rows that an SM takes (of n / SMs).  FP64
- *                     multiply-adds when a column holds Inf or NaN;
+ *                     multiply-adds when a column holds Inf or NaN, values from
+ *                     2^1017 up, or in an SM's rows nothing from 2^-895 up but
+ *                     not only zeros;
  *   PLHR_GRAM_F32     FP32 blocks, FP32 products on the FP32 pipes, sums
  *                     folded into double-FP32 every 32 rows;
  *   PLHR_GRAM_DW      FP64 blocks, the form of the mixed solve's FP64-storage

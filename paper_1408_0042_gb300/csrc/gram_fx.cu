@@ -43,9 +43,9 @@
 // shifted to the new exponents and the CTA goes on.  So the precision is relative to
 // the columns' norms (what the Cholesky factorisation of a Gram matrix needs), not to
 // each pair of entries.
-// A column holding Inf or NaN and a wait that times out set the CTA's flag: the
-// plain FP64 kernel, which is launched behind this one and returns at once
-// otherwise, then redoes the Grams.
+// A column holding Inf or NaN or values outside the exponents' range (kExpFloor,
+// kExpTop) and a wait that times out set the CTA's flag: the plain FP64 kernel, which
+// is launched behind this one and returns at once otherwise, then redoes the Grams.
 //
 // Tiles (mp = m rounded up to 16).  A step of 32 rows is one K-major panel of
 // operand rows per digit.  [Z_k; Q_k] with Z_l, 128 x mp x 16, gives Z^T Z and
@@ -93,7 +93,11 @@ constexpr int kFxMeta = 10240;
 constexpr int kLdD = 33;                       // staging of 32 columns of sums
 constexpr int kFxSmem = kFxOperand + kFxMeta + 128 * kLdD * 8;
 constexpr int kIssuers = 4;
-constexpr int kExpFloor = 128;                 // exponents start here: smaller values (below 2^-894) count as zero
+// Exponents start at kExpFloor: a share of a column that has nothing from 2^-895 up, but
+// not only zeros, is left to k_gram, and so are values from 2^1017 up, whose column
+// factors could leave the range that their products with the column scales keep
+constexpr int kExpFloor = 128;
+constexpr int kExpTop = 0x7f8;
 constexpr long long kFxWait = 4LL << 30;       // about 2 s
 
 struct FxCols {
@@ -470,12 +474,19 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                 mq = max(mq, exp_field(qv[i]));
             }
         };
-        // raise the exponents of the warp's columns to the loaded values (Inf and NaN
-        // set the flag and leave them alone); whether this thread's had to
+        // families (bits) of the thread's column with a value other than zero so far, while
+        // the exponent is still the floor
+        int low = 0;
+        auto note_low = [&](int f, const double* v) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) low |= (__double_as_longlong(v[i]) << 1) != 0 ? f : 0;
+        };
+        // raise the exponents of the warp's columns to the loaded values (too large ones,
+        // Inf and NaN set the flag, Inf and NaN leave them alone); whether this thread's had to
         auto raise = [&]() -> bool {
             const bool up = mz >= ez || mu >= eu || mq >= eq;
             if (!__any_sync(0xffffffffu, up)) return false;
-            if (mz == 0x7ff || mu == 0x7ff || mq == 0x7ff) bad = true;
+            if (max(mz, max(mu, mq)) >= kExpTop) bad = true;
             auto one = [&](int& e, int mx, int at_col) {
                 int x = mx >= e && mx != 0x7ff ? mx + room : e;
                 for (int o = 4; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
@@ -516,6 +527,11 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
             if (!last) {
                 if (conv) prepare();
                 if (convw) grow = raise();
+                if (conv && min(ez, min(eu, eq)) == kExpFloor) {
+                    if (ez == kExpFloor) note_low(1, z);
+                    if (eu == kExpFloor) note_low(2, a);
+                    if (eq == kExpFloor) note_low(4, qv);
+                }
                 // the MMAs of two steps ago have read this panel
                 if (st >= 2) w = tc::mbar_wait(&S.done[st & 1], (uint32_t)(((st >> 1) - 1) & 1), kFxWait);
                 unsigned char* pan = smem + (st & 1) * panel_of(mp);
@@ -577,6 +593,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
             pending = true;
             ++issued;
         }
+        if ((low & 1 && ez == kExpFloor) || (low & 2 && eu == kExpFloor) || (low & 4 && eq == kExpFloor)) bad = true;
         if (!ok && tid == 0) {       // let the issuing warps go
             S.stop = 1;
             tc::mbar_arrive(&S.full[issued & 1]);
