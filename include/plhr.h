@@ -320,7 +320,8 @@ plhr_status plhr_eigval_grad(int64_t n, int k, const double* V, int64_t ldv, con
  * written to *iterations when non-null).  Pairs with |lam_c - lam_j| <= 1e-12 max(1,
  * |lam_0|) contribute no in-block term (a repeated eigenvalue has no
  * eigenvector derivative inside its eigenspace).  1 <= k <= 16.  The call
- * synchronises the stream (it reads two inner products per iteration) and
+ * synchronises the stream (it reads two inner products per iteration; on
+ * return grad is complete and V, G may be reused) and
  * allocates its own device workspace (9 n x k doubles).  PLHR_EINVAL on bad
  * arguments, PLHR_ENOMEM when the workspace cannot be allocated, PLHR_ENAN
  * on a non-finite inner product, PLHR_ENOTCONV when maxit is reached (grad

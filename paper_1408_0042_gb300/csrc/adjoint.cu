@@ -142,7 +142,7 @@ extern "C" plhr_status plhr_eigvec_adjoint(const plhr_op* A, plhr_prec* T, int k
     struct Free {
         double* p;
         cudaStream_t s;
-        ~Free() { ws_free(p, s); }
+        ~Free() { cudaStreamSynchronize(s); ws_free(p, s); }   // no return before the stream's work is done
     } fr{ws, s};
     double* q = ws;
     double *x = q; q += nk;
@@ -316,6 +316,7 @@ extern "C" plhr_status plhr_eigvec_adjoint(const plhr_op* A, plhr_prec* T, int k
     count_launches(2);
     PLHR_TRY_CUDA(cudaGetLastError());
     if (iterations) *iterations = itn;
+    PLHR_TRY_CUDA(cudaStreamSynchronize(s));   // a fault of the kernels since the last inner product is this call's
     if (!converged) {
         set_error("plhr_eigvec_adjoint: MINRES did not reach tol in %d iterations", maxit);
         return PLHR_ENOTCONV;
