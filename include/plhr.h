@@ -24,6 +24,12 @@
  *     failing CUDA call gives PLHR_ECUDA (plhr_last_error() has the text).
  *   - Every entry point needs the CUDA device that holds the pointers to be
  *     current on the calling thread.
+ *   - plhr_gram, plhr_tharm_extract and plhr_eigvec_adjoint take their workspace
+ *     from a memory pool of the library, which keeps at most 64 MiB per device
+ *     between calls.  The pool is given back when the process's last operator or
+ *     preconditioner is destroyed (a workspace still in use on a stream then,
+ *     with the next synchronisation); a program that holds none gives it back
+ *     by creating and destroying one.
  */
 #ifndef PLHR_H
 #define PLHR_H

@@ -41,7 +41,15 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
+bool g_keeps[kMaxDevices] = {false};   // the pool's release threshold is kPoolKeep, not 0
 std::atomic<int> g_live{0};
+
+void set_keep(int dev, bool keep) {
+    if (g_keeps[dev] == keep) return;
+    unsigned long long bytes = keep ? kPoolKeep : 0;
+    if (cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &bytes) == cudaSuccess) g_keeps[dev] = keep;
+    else cudaGetLastError();
+}
 
 // the current device's pool, created on its first use; nullptr when there is none
 cudaMemPool_t pool_of_device() {
@@ -54,14 +62,13 @@ cudaMemPool_t pool_of_device() {
         pr.location.type = cudaMemLocationTypeDevice;
         pr.location.id = dev;
         cudaMemPool_t pool = nullptr;
-        unsigned long long keep = kPoolKeep;
         if (cudaMemPoolCreate(&pool, &pr) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
         g_pool[dev] = pool;
     }
+    set_keep(dev, true);
     return g_pool[dev];
 }
 }  // namespace
@@ -86,8 +93,11 @@ LiveObject::LiveObject() { g_live.fetch_add(1); }
 LiveObject::~LiveObject() {
     if (g_live.fetch_sub(1) != 1) return;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (cudaMemPool_t pool : g_pool)
-        if (pool) cudaMemPoolTrimTo(pool, 0);
+    for (int dev = 0; dev < kMaxDevices; ++dev)
+        if (g_pool[dev]) {
+            set_keep(dev, false);   // a release that is still queued leaves the pool with the next synchronisation
+            cudaMemPoolTrimTo(g_pool[dev], 0);
+        }
 }
 
 }  // namespace plhr

@@ -88,7 +88,8 @@ int sm_count();
 // of the library's own: freed blocks stay in the pool up to kPoolKeep bytes
 // per device, so that a call does not map and unmap device memory each time
 // (about 100 us per allocation).  The pool gives what it keeps back to the
-// device when the last operator or preconditioner is destroyed, and when an
+// device when the last operator or preconditioner is destroyed (what is still
+// queued on a stream then, with the next synchronisation), and when an
 // allocation fails (which is then tried again).
 constexpr unsigned long long kPoolKeep = 64ull << 20;
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
