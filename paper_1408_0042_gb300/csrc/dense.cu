@@ -757,9 +757,9 @@ struct DenseState {
     int ints[8];              // [0] kept columns, [1] of V, [3] selected units, [6] stop, [7] pencil's verdict
 };
 
-// Yre, Yim (MAXM^2 each; MAXM^2 unused), then the saved state
+// Yre, Yim (MAXM^2 each), then the saved state
 constexpr int MAXKP = 16;
-constexpr size_t kWorkMainDoubles = 3 * (size_t)MAXM * MAXM;
+constexpr size_t kWorkMainDoubles = 2 * (size_t)MAXM * MAXM;
 constexpr size_t kDenseWorkDoubles = kWorkMainDoubles + (sizeof(DenseState) + sizeof(double) - 1) / sizeof(double);
 
 __device__ __forceinline__ DenseState* state_of(const DenseArgs& a) {
@@ -1321,10 +1321,7 @@ __global__ void __launch_bounds__(128) k_finish(DenseArgs a) {
 
 }  // namespace
 
-// Yre, Yim (MAXM^2 each; MAXM^2 unused) and the shared-memory state passed
-// between the launches.
 size_t dense_work_doubles() { return kDenseWorkDoubles; }
-static_assert(kWorkMainDoubles >= 3 * (size_t)MAXM * MAXM, "dense scratch layout");
 
 cudaError_t dense_extract(const DenseArgs& a, cudaStream_t s) {
     size_t shm = sizeof(PencilShm);
@@ -1597,7 +1594,7 @@ extern "C" plhr_status plhr_tharm_extract(int m, int kp, int nv, const double* G
 namespace {
 
 // Scratch of the projected eigensolve for the largest supported basis
-// (m = 64): three 64 x 64 arrays and the saved state, about 262 KiB.  Every
+// (m = 64): two 64 x 64 arrays and the saved state, about 230 KiB.  Every
 // GPU that loads the library holds this array until the process exits.
 constexpr size_t kNoAllocScratchDoubles = plhr::kDenseWorkDoubles;
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];

@@ -115,7 +115,6 @@ __device__ __forceinline__ float pow2_inverse_of(float x) {
     return __int_as_float((254 - k) << 23);
 }
 
-__device__ __forceinline__ float dw_abs_hi(dw a) { return fabsf(a.hi); }
 __device__ __forceinline__ bool dw_is_zero(dw a) { return a.hi == 0.0f; }
 
 // conversions (FP64 instructions: use outside inner loops)
