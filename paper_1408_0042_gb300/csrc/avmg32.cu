@@ -424,8 +424,10 @@ __global__ void __launch_bounds__(kT) k_restrict_line(Lv gf, Lv gc, int lin, con
 
 // Linear restriction in 3D, four coarse lines (2 along y x 2 along z) per CTA: a fine
 // value is read 2.25 times instead of 4, six independent loads at a time instead of
-// one after the other (128^3 x 32: 127 -> 62 us, 64^3: 23 -> 11; where it leaves
-// fewer CTAs than SMs, one line a CTA is faster: 32^3 8 us against 6).
+// one after the other (128^3 x 32: 127 -> 62 us, 64^3: 23 -> 11), at any length of a line
+// (V-cycles of 64 x 64 lines of 64 to 1024 values 51 to 84 us before, 47 to 80).  Where it
+// leaves fewer CTAs than SMs, one line a CTA is faster (32^3 8 us against 6; V-cycles
+// of 32 x 32 and 40 x 40 lines 39 to 56 us against 41 to 58).
 constexpr int kQuadT = 512;
 template <int VW>
 __global__ void __launch_bounds__(kQuadT) k_restrict_quad(Lv gf, Lv gc, const float* __restrict__ f,
@@ -669,7 +671,7 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, bool v4, const Tr* r, in
     }
     const size_t quad = 4 * sizeof(float) * L.g.nx * nc;
     cudaError_t e;
-    if (d3 && H.linear && quad <= kQuadSmemMax && Lc.g.nz <= 65535 && L.g.nx * nc >= kQuadT &&
+    if (d3 && H.linear && quad <= kQuadSmemMax && Lc.g.nz <= 65535 &&
         ((Lc.g.ny + 1) / 2) * ((Lc.g.nz + 1) / 2) >= sm_count()) {
         auto kern = v4 ? k_restrict_quad<4> : k_restrict_quad<1>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQuadSmemMax);

@@ -336,7 +336,9 @@ __global__ void __launch_bounds__(kT) k_restrict_line(Ld gf, Ld gc, int lin, con
 // Linear restriction in 3D, four coarse lines (2 along y x 2 along z) per CTA: a fine
 // value is read 2.25 times instead of 4, six independent loads at a time instead of
 // one after the other.  The weights are 1 and 3, the power of two comes last
-// (96 x 80 x 64 x 11: 69 -> 27 us).
+// (96 x 80 x 64 x 11: 69 -> 27 us).  At any length of a line and any number of them that
+// fits: V-cycles of 64 x 64 lines of 64 to 1024 values 68 to 236 us with one line a CTA,
+// 64 to 216 with four, of 16 x 16 lines of 64 to 2048 values 40 to 92 and 39 to 76.
 constexpr int kQuadT = 512;
 constexpr size_t kQuadSmemMax = 96 * 1024;
 __global__ void __launch_bounds__(kQuadT) k_restrict_quad(Ld gf, Ld gc, const dw* __restrict__ f,
@@ -589,8 +591,7 @@ cudaError_t vcycle(const MGHierarchy& H, int l, int nc, const dw* r, dw* out, co
     }
     const size_t quad = 4 * sizeof(dw) * L.g.nx * nc;
     cudaError_t e;
-    if (d3 && H.linear && quad <= kQuadSmemMax && Lc.g.nz <= 65535 && L.g.nx * nc >= kQuadT &&
-        ((Lc.g.ny + 1) / 2) * ((Lc.g.nz + 1) / 2) >= sm_count()) {
+    if (d3 && H.linear && quad <= kQuadSmemMax && Lc.g.nz <= 65535) {
         e = cudaFuncSetAttribute(k_restrict_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQuadSmemMax);
         if (e != cudaSuccess) return e;
         k_restrict_quad<<<dim3((unsigned)((Lc.g.ny + 1) / 2), (unsigned)((Lc.g.nz + 1) / 2)), kQuadT, quad, s>>>(
