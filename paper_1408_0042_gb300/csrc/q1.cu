@@ -24,7 +24,7 @@
 // below it (a thread walks up the z axis with its face), and an element's
 // products leave through the same butterflies: about 36 FP64 operations per
 // node instead of the 72 multiply-adds of 8 cells times 8 corners, with the mass
-// product 47 instead of 130 (64^3 elements, 9 columns: 499 -> 277 us; the tiles'
+// product 47 instead of 130 (64^3 elements, 9 columns: 499 -> 271 us; the tiles'
 // repeated faces, partly filled warps and the SMs without a CTA make the pipe's
 // 188 us 245).
 //
@@ -172,6 +172,12 @@ Q1Geo q1geo(const Grid& g) { return {g.nx, g.ny, g.nz, g.h, g.cell}; }
 // times the planes it passes (one more than it puts out) times the rounds of
 // CTAs over the SMs.  A face row and column and an element plane are repeated
 // per tile, partly filled warps and last rounds cost as much as full ones.
+// Candidates: edges whose faces fill whole warps or nearly (16^2, 13^2, 11^2, 9^2,
+// 18^2 faces) at 1 to 4 columns.  With edge 15 alone 40^3 x 2 takes 33 us against 25,
+// without 17 64^3 x 9 takes 277 against 271; edges 6, 20, 24, 31 win nothing.  Wide
+// blocks take 3 or 4 columns (longer runs of memory), few columns make more CTAs
+// on small grids: 48 x 40 x 56 x 5 84 us with 3 or 4 only, 68 with 1 to 4; up to 8
+// columns win nothing.
 Q1Tile q1_tile(const Grid& g, int nc, dim3& grid, int& threads, size_t& smem) {
     auto even = [](int64_t n, int64_t most) {
         const int64_t parts = (n + most - 1) / most;
@@ -181,10 +187,13 @@ Q1Tile q1_tile(const Grid& g, int nc, dim3& grid, int& threads, size_t& smem) {
     Q1Tile best{};
     double least = 0.0;
     int64_t ctas = 0, segs = 0;
-    for (int cmax = nc < 4 ? nc : 4; cmax >= (nc < 3 ? nc : 3); --cmax)
+    for (int cmax = nc < 4 ? nc : 4, last = 0; cmax >= 1; --cmax) {
+        const int cols = even(nc, cmax);
+        if (cols == last) continue;
+        last = cols;
         for (int edge : {15, 12, 10, 8, 17}) {
             Q1Tile k;
-            k.cols = even(nc, cmax);
+            k.cols = cols;
             k.chunks = (nc + k.cols - 1) / k.cols;
             k.tx = even(g.nx, edge);
             k.ty = even(g.ny, edge);
@@ -205,6 +214,7 @@ Q1Tile q1_tile(const Grid& g, int nc, dim3& grid, int& threads, size_t& smem) {
                 if (k.tz <= 4) break;
             }
         }
+    }
     grid = dim3((unsigned)ctas, (unsigned)segs);
     const int cells = (best.tx + 1) * (best.ty + 1) * best.cols;
     threads = (cells + 31) / 32 * 32;
