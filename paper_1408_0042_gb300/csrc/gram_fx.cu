@@ -25,17 +25,17 @@
 // their largest, accumulate exactly in FP32 tensor memory.  Levels 4 to 6 share an
 // accumulator, which drops what is below 2^-24 of its content with each MMA.  At the
 // end of a period the accumulators are read back as integers into 64-bit sums
-// in units of 2^-36 of the leading digit product (2^-54 of 2^E 2^E').
+// in units of 2^-35 of the leading digit product (2^-53 of 2^E 2^E').
 //
 // Accuracy.  On columns whose entries are of one size, such as trial bases, an entry is
 // correct to a few 2^-53 of the column norms: 2e-16 to 9e-16 of |x| |y| at 40,000 to
 // 2,097,152 rows (FP64 multiply-adds 2e-16 to 1.3e-15, double-word ones 5e-15 to
 // 2e-11).  A column with few large entries and a long tail of equal low digits loses
 // up to 2^-40 of the product of the largest entries per 128 rows of an SM (128 MMAs
-// at one unit of the shared accumulator); measured with one entry 1 and 10^-3 to
-// 10^-6 elsewhere at 2,097,152 rows: 1e-13, 2.4e-12 (10^-4), 9e-14 where FP64
-// multiply-adds lose 1e-13, 6e-13, 6e-13.  Without level 6, which has 2 d_1 d_5 and
-// 2 d_2 d_4 of one sign there, it was 1.7e-12, 6.5e-12, 5e-13.
+// at one unit of the shared accumulator); measured with one entry 1 and 10^-3, 10^-4 or
+// 10^-6 elsewhere at 2,097,152 rows: 1e-13, 2.4e-12, 2e-13 where FP64 multiply-adds
+// lose 1e-13, 6e-13, 6e-13 (without all of level 6, which has 2 d_1 d_5 and 2 d_2 d_4 of
+// one sign there: 1.7e-12, 6.5e-12, 5e-13).
 //
 // Exponents.  E is kept per column and CTA: the largest exponent met so far
 // plus two, in long runs from 32 rows spread over the CTA's share on.
@@ -78,7 +78,10 @@ constexpr int kFxThreads = kFxConv + 128;      // and a warpgroup that issues th
 constexpr int kFxK = 32;                       // rows per step
 constexpr int kMaxPeriod = 4;                  // steps per period
 constexpr int kDigits = 6;
-constexpr int kUnit = 36;                      // the 64-bit sums are in units of 2^-kUnit of the leading digit product
+// the 64-bit sums are in units of 2^-kUnit of the leading digit product: a period adds at
+// most 2^58 of them, so a CTA writes its sums out where one may pass 2^62 (at 2^-36 the
+// 128^3 trial basis does so: 2.68 ms against 2.65 at m = 64)
+constexpr int kUnit = 35;
 constexpr int kCore = 128;                     // core matrix: 8 rows x 16 bytes
 // A step's panel: the U digits between two blocks of zeros (per core column of 8
 // rows of the step: [0 | U0 | .. | U5 | 0], 8 mp operand rows), then per digit a
@@ -358,7 +361,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
         };
         // Add the accumulators of the MMAs issued so far (the last of them for step
         // st) to the integers; false when the wait timed out.  full: some integer is
-        // within a factor 4 of its range.
+        // from 2^62 up.
         bool full = false;
         auto drain = [&](int st) -> bool {
             if (!tc::mbar_wait(&S.done[st & 1], (uint32_t)((st >> 1) & 1), kFxWait)) return false;
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     }
                 }
             }
-            full = top >= 1u << 29;
+            full = top >= 1u << 30;
             tc::fence_before_sync();
             return true;
         };

@@ -40,8 +40,8 @@ def _error(plhr, Z):
 def test_products_of_outer_digits_are_kept(plhr):
     """A tail with the digits 1 and 5 only, both 255: its products are of levels 2, 6 and
     10, and those of level 6, 2^17 2^-72 a row, all have one sign.  Level 6 sums exactly
-    (255 256 2 128 < 2^24); left are a rounding of half a unit of 2^-54 at the end of
-    each of the 32 periods of 128 rows and the few of the result: below 2^-43."""
+    (255 256 2 128 < 2^24); left are a rounding of half a unit of 2^-53 at the end of
+    each of the 32 periods of 128 rows, 2^-43 of the largest entries and 2^-43.3 of the norms, and the few of the result."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     periods = 32
     Z = np.zeros((sms * 128 * periods, 2))
@@ -56,7 +56,7 @@ def test_long_tails_stay_within_the_stated_bound(plhr, tail):
     """The stated bound: 2^-40 of the product of the largest entries for every 128 rows
     of an SM.  With tails below 2^-9 of the largest entry the levels above 4 are exact
     and the sum of levels 4 to 6 stays below 2^24 units of 2^-54; each of the 128 MMAs
-    of a period may lose one unit, and the read-back half of one: 129 2^-54 2^6."""
+    of a period may lose one unit, and the read-back half of one of 2^-53: 129 2^-54 2^6."""
     n = 300000
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     rng = np.random.default_rng(5)
