@@ -44,6 +44,14 @@ cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
 bool g_keeps[kMaxDevices] = {false};   // the pool's release threshold is kPoolKeep, not 0
 std::atomic<int> g_live{0};
 
+// Creating, trimming and setting up a pool touch no stream, but count as unsafe while a
+// stream is captured (by this or another thread) and would invalidate the capture
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 void set_keep(int dev, bool keep) {
     if (g_keeps[dev] == keep) return;
     unsigned long long bytes = keep ? kPoolKeep : 0;
@@ -56,6 +64,7 @@ cudaMemPool_t pool_of_device() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
     std::lock_guard<std::mutex> lk(g_pool_mu);
+    RelaxedCapture relaxed;
     if (!g_pool[dev]) {
         cudaMemPoolProps pr{};
         pr.allocType = cudaMemAllocationTypePinned;
@@ -79,7 +88,10 @@ cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s) {
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        cudaMemPoolTrimTo(pool, 0);
+        {
+            RelaxedCapture relaxed;
+            cudaMemPoolTrimTo(pool, 0);
+        }
         e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     }
     return e;
@@ -93,6 +105,7 @@ LiveObject::LiveObject() { g_live.fetch_add(1); }
 LiveObject::~LiveObject() {
     if (g_live.fetch_sub(1) != 1) return;
     std::lock_guard<std::mutex> lk(g_pool_mu);
+    RelaxedCapture relaxed;
     for (int dev = 0; dev < kMaxDevices; ++dev)
         if (g_pool[dev]) {
             set_keep(dev, false);   // a release that is still queued leaves the pool with the next synchronisation
