@@ -57,9 +57,9 @@ def _peaks():
 FP64_PEAK_TFLOPS = 1.25
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_gram_fx launch
-# (n = 262,144, m = 36: 231.9 MB read, 6.0 MB written), i.e. bytes per (row x trial column); the traffic
-# grows in proportion to n m.
-GRAM_DRAM_BYTES_PER_ROW_COL = 237.9e6 / (262144 * 36)
+# (n = 262,144, m = 64: 409.4 MB read, 4.9 MB written; profiles/kernels.md), i.e. bytes per
+# (row x trial column); the traffic grows in proportion to n m.
+GRAM_DRAM_BYTES_PER_ROW_COL = 414.3e6 / (262144 * 64)
 
 
 class ClockSampler:
@@ -173,9 +173,9 @@ def _fp32_simt_peak_tflops(sm_mhz):
 
 
 PHASE_KERNELS = {
-    "stencil": "k_lap_axpby / k_lap_shifts (FP64) and k_lap32 (FP32) stencil products",
+    "stencil": "k_lap_fx (FP64, small blocks k_lap_axpby / k_lap_shifts) and k_lap32 (FP32) stencil products",
     "preconditioner": "AV-MG V-cycle kernels (FP64 form; double-word in the mixed form's FP64 phase)",
-    "gram": "k_gram_fx (tcgen05 multi-Gram on exact fixed-point slices, FP64 accuracy)",
+    "gram": "k_gram_fx (tcgen05 multi-Gram on fixed-point slices, FP64-class accuracy)",
     "update": "k_update (FP64; k_update_dw double-word in the mixed form's FP64 phase)",
     "residual": "k_residual (residual block and column norms)",
     "preconditioner_f32": "FP32 AV-MG V-cycle kernels",
@@ -192,13 +192,13 @@ def _rooflines(prof, peaks, sm_max_mhz, mixed, tensor_cores=True):
     tensor rate as a second figure: the double-word multiply-add costs 13
     FP32 instructions for 2 FP64-equivalent flops (roof = FP32 lane rate / 13),
     the FP64 kernels run at the FP64 rate of the profiling recipe, and the
-    tensor-core Grams execute six (FP32 form) or 22 (FP64 and double-word forms)
+    tensor-core Grams execute six (FP32 form) or 26 (FP64 and double-word forms)
     BF16 products per useful product."""
     out = []
     fp32_peak = _fp32_simt_peak_tflops(sm_max_mhz or 2070.0)
     dw_peak = fp32_peak / 13.0
     alu = {
-        "gram": ("BF16 tensor rate (22 digit products per product)", peaks["bf16_tflops"], 22.0),
+        "gram": ("BF16 tensor rate (26 digit products per product)", peaks["bf16_tflops"], 26.0),
         "update": ("double-word FP32-pipe roof" if mixed else "FP64 rate", dw_peak if mixed else FP64_PEAK_TFLOPS,
                    1.0),
         "gram_f32": (("BF16 tensor rate (6 slice products per product)", peaks["bf16_tflops"], 6.0) if tensor_cores
@@ -350,7 +350,7 @@ def run_ours(args, world, rank, local):
             per = GRAM_DRAM_BYTES_PER_ROW_COL
             m_avg = dom["bytes_per_call"] / (24.0 * n)
             dom["traffic"] = per * n * m_avg
-            dom["traffic_note"] = ("ncu dram__bytes_read + write of one k_gram_fx launch (n = 262,144, m = 36), "
+            dom["traffic_note"] = ("ncu dram__bytes_read + write of one k_gram_fx launch (n = 262,144, m = 64), "
                                    "scaled by n m to this run's average launch (n = %d, m = %.1f)" % (n, m_avg))
     dense = prof.get("dense", {})
     dense_stage = {"ms_per_iteration": dense["ms"] / dense["calls"] if dense.get("calls") else None,
@@ -576,6 +576,15 @@ GRAD_METRIC = ("seconds per forward + backward: k = 8 eigenpairs nearest sigma a
                "sum_k w_k lambda_k + sum_k |m (.) v_k|^2, 64^3 Hamiltonian")
 
 
+def _folded_madds(N):
+    """Multiply-adds of one periodic TPA axis transform of a line of N points:
+    a square product per parity class, two classes (odd N) or four (even N)."""
+    even, odd = N // 2 + 1, (N - 1) // 2
+    if N % 2 or N < 4:
+        return even ** 2 + odd ** 2
+    return sum(((q + r) // 2) ** 2 for q in (even, odd) for r in (0, 1))
+
+
 def run_grad(args, world, rank, local):
     """The differentiation workload: a step is the forward solve (TPA-
     preconditioned block PLHR, FP64, tol 1e-10) plus the backward pass
@@ -678,17 +687,20 @@ def run_grad(args, world, rank, local):
         e2e.append(time.perf_counter() - t0)
     e2e_s = _max_over_ranks(statistics.mean(e2e), world)
 
-    # rooflines of the phases the library times; the TPA application is dense
-    # per-axis transforms in double-word arithmetic: 2 (forward, inverse) x 2
-    # flops x (nx + ny + nz) per element (grid point x column)
+    # rooflines of the phases the library times; the TPA application is one
+    # product per parity class and axis in double-word arithmetic, forward and
+    # inverse (grid point x column elements, 2 flops a multiply-add); the Gram
+    # takes 26 BF16 digit products per product
+    peaks = _peaks()
     fp64 = FP64_PEAK_TFLOPS
     dw_peak = _fp32_simt_peak_tflops(clocks.get("sm_max_mhz") or 2070.0) / 13.0
-    per_elem = 4.0 * sum(dims)
+    per_elem = sum(4.0 * _folded_madds(N) / N for N in dims)
     roofs = []
     for ph, kernel, per, peak, src in (
             ("preconditioner", "k_axis (TPA transforms, double-word)", per_elem * 1e-12, dw_peak,
              "FP32 lanes x clock / 13 x 2 flops (double-word multiply-add = 13 FP32 instructions)"),
-            ("gram", "k_gram (FP64 multi-Gram)", 1e-12, fp64, "nominal FP64 rate of the profiling recipe"),
+            ("gram", "k_gram_fx (tcgen05 multi-Gram on fixed-point slices)", 26e-12, peaks["bf16_tflops"],
+             "%s (MEASURED_PEAKS.json bf16_tflops), 26 digit products per product" % peaks["src"]),
             ("update", "k_update (FP64)", 1e-12, fp64, "nominal FP64 rate of the profiling recipe")):
         d = prof.get(ph)
         if not d or d["ms"] <= 0 or d["work"] <= 0:
@@ -745,11 +757,11 @@ def grad_cpu_baseline(gpu_iterations):
 
 
 # Iterations of the all-FP64 GPU form to relative residual 1e-8 on the 128^3
-# workload (293, measured on GB300 by this bench's fp64 leg); the oracle runs
+# workload (279, measured on GB300 by this bench's fp64 leg); the oracle runs
 # the same FP64 iteration, and its own count would take over an hour of host
 # time to measure, so the reference arm scales its per-iteration time by the
 # GPU's count.
-GPU_F64_ITERATIONS_TO_TOL = 293
+GPU_F64_ITERATIONS_TO_TOL = 279
 
 
 def run_reference(args, world, rank, local):
