@@ -347,9 +347,9 @@ cudaError_t multi_gram_b(int64_t n, int nb, const Blk<const double>* Z, const Bl
     int blocks = reduce_blocks();
     int* flags = nullptr;
     if (!BZ) {
-        // B = I: exact slices on the tensor cores at every n and m (262,144 rows,
-        // m = 36: 302 us against 2.36 ms); k_gram then only works on columns with Inf
-        // or NaN.  With a B family it is the only form.
+        // B = I: fixed-point slices on the tensor cores at every n and m (262,144 rows,
+        // m = 36: a call 370 us against 2.64 ms); k_gram then only works on columns with
+        // Inf, NaN or values at the ends of the range.  With a B family it is the only form.
         cudaError_t e = gram_fx_launch(n, nb, Z, AZ, Q, sigma, colscale, partial, &blocks, &flags, s);
         if (e != cudaSuccess) return e;
     }

@@ -57,7 +57,7 @@ plhr_status plhr_gram(int form, int64_t n, int nb, const int* ncols, const void*
             ab[b] = {static_cast<const double*>(AZ[b]), ldaz[b], ncols[b]};
             if (Q) qb[b] = {static_cast<const double*>(Q[b]), ldq[b], ncols[b]};
         }
-        // both forms are the exact-slice tensor-core Gram
+        // both forms are the fixed-point tensor-core Gram
         PLHR_TRY_CUDA(multi_gram(n, nb, zb.data(), ab.data(), Q ? qb.data() : nullptr, sigma, colscale, partial, out,
                                  s));
     } else {

@@ -1,5 +1,5 @@
 // The three projected Grams of FP64 blocks on the tensor cores (tcgen05), by
-// exact fixed-point slices.
+// fixed-point slices.
 //
 // With the trial basis Z (m <= 64 columns), its image A Z and the T-harmonic
 // images Q, U = A Z - sigma Z and column scales D,
@@ -60,13 +60,13 @@
 // stands still for the time they take); 16 warps convert, and read the
 // accumulators back every 128 rows.  A converting warp takes 4 columns, all 32
 // rows, so that it agrees on their exponents by shuffles; the next step's
-// values are in flight in registers meanwhile.  The conversion, about 40
-// integer and FP32 instructions per value, is what binds: 4.6k of 9k cycles
-// per step, the rest loads, the barrier and the read-back.
+// values are in flight in registers meanwhile.  A step takes about 12k cycles: the
+// conversion, about 40 integer and FP32 instructions per value, 4.6k of them, the
+// rest loads, the barrier and a period's share of the read-back.
 //
-// Measured on GB300 on trial bases of a Laplacian: m = 36, 262,144 rows 302 us
-// (FP64 multiply-adds 2.36 ms, bound by the FP64 pipe); m = 64, 2,097,152 rows
-// 2.47 ms (double-word multiply-adds on the FP32 pipes 9.45 ms).
+// Measured on GB300 on trial bases of a Laplacian: m = 36, 262,144 rows 370 us a call
+// (FP64 multiply-adds 2.64 ms, bound by the FP64 pipe); m = 64, 2,097,152 rows
+// 2.56 ms (double-word multiply-adds on the FP32 pipes 9.45 ms).
 #include "blockops.h"
 #include "tc.h"
 
