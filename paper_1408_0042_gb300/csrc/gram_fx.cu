@@ -118,6 +118,7 @@ struct FxMeta {
     // 2^(exponent - 1022)
     int e[192];
     int en[192];
+    int low[192];             // met a value other than zero while the exponent was the floor
     double fac[192];
     FxCols cols;
 };
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
         S.cols.p[f][j] = C.p[f][j];
         S.cols.ld[f][j] = C.ld[f][j];
         S.e[t] = S.en[t] = kExpFloor;
+        S.low[t] = 0;
     }
     // the zero block, padding columns and what A reads past a panel stay zero
     for (int t = tid; t < kFxOperand / 16; t += kFxThreads) reinterpret_cast<uint4*>(smem)[t] = make_uint4(0, 0, 0, 0);
@@ -430,13 +432,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     const int y = (cc >> 3) * ncol + c + (cc & 7);
                     if (y >= m || c + (cc & 7) >= ncol) continue;
                     // units of 2^-kUnit of a leading digit product; a column's leading digit is
-                    // in units of 2^-9 2^(exponent - 1022)
+                    // in units of 2^-9 2^(exponent - 1022).  One factor after the other: the product
+                    // of two factors can leave the range (large column scales) where the sum is 0.
                     constexpr double unit = 1.0 / (double)(1ull << (18 + kUnit));
                     if (u) {
                         // even levels in row i, odd ones in row mp + i; the upper triangle, mirrored
                         if (i >= m || i > y) continue;
                         const double v = (D[i * kLdD + cc] + D[(mp + i) * kLdD + cc] * 0x1p-9) * unit *
-                                         (S.fac[2 * mp + i] * S.fac[mp + y]);
+                                         S.fac[2 * mp + i] * S.fac[mp + y];
                         double* o = out + m * m;
                         const double s = first ? v : o[i * m + y] + v;
                         o[i * m + y] = s;
@@ -444,7 +447,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                     } else {
                         const int x = i < mp ? i : i - mp;
                         if (i >= 2 * mp || x >= m) continue;
-                        const double v = D[i * kLdD + cc] * unit * (S.fac[i] * S.fac[y]);
+                        // (x, y) and (y, x) of Z^T Z are rounded alike
+                        const int a = i < mp ? min(x, y) : i, b = i < mp ? max(x, y) : y;
+                        const double v = D[i * kLdD + cc] * unit * S.fac[a] * S.fac[b];
                         double* o = out + (i < mp ? 0 : 2 * m * m) + x * m + y;
                         *o = first ? v : *o + v;
                     }
@@ -477,12 +482,12 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                 mq = max(mq, exp_field(qv[i]));
             }
         };
-        // families (bits) of the thread's column with a value other than zero so far, while
-        // the exponent is still the floor
-        int low = 0;
-        auto note_low = [&](int f, const double* v) {
+        // the thread's values of column at_col are not all zero
+        auto note_low = [&](const double* v, int at_col) {
+            bool any = false;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) low |= (__double_as_longlong(v[i]) << 1) != 0 ? f : 0;
+            for (int i = 0; i < 4; ++i) any |= (__double_as_longlong(v[i]) << 1) != 0;
+            if (any) S.low[at_col] = 1;
         };
         // raise the exponents of the warp's columns to the loaded values (too large ones,
         // Inf and NaN set the flag, Inf and NaN leave them alone); whether this thread's had to
@@ -531,9 +536,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
                 if (conv) prepare();
                 if (convw) grow = raise();
                 if (conv && min(ez, min(eu, eq)) == kExpFloor) {
-                    if (ez == kExpFloor) note_low(1, z);
-                    if (eu == kExpFloor) note_low(2, a);
-                    if (eq == kExpFloor) note_low(4, qv);
+                    if (ez == kExpFloor) note_low(z, j);
+                    if (eq == kExpFloor) note_low(qv, mp + j);
+                    if (eu == kExpFloor) note_low(a, 2 * mp + j);
                 }
                 // the MMAs of two steps ago have read this panel
                 if (st >= 2) w = tc::mbar_wait(&S.done[st & 1], (uint32_t)(((st >> 1) - 1) & 1), kFxWait);
@@ -596,7 +601,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_gram_fx(int64_t n, int m, int
             pending = true;
             ++issued;
         }
-        if ((low & 1 && ez == kExpFloor) || (low & 2 && eu == kExpFloor) || (low & 4 && eq == kExpFloor)) bad = true;
+        if (tid < 3 * mp && S.low[tid] && S.e[tid] == kExpFloor) bad = true;
         if (!ok && tid == 0) {       // let the issuing warps go
             S.stop = 1;
             tc::mbar_arrive(&S.full[issued & 1]);

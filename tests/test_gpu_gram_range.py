@@ -59,3 +59,23 @@ def test_products_across_the_range(plhr):
     for g, f in zip(G, (1.0, 6.25, -2.5)):
         assert abs(g[0, 1] / (f * ref * 2.0 ** 21) - 1.0) <= 2.0 ** -46
         assert np.isinf(g[0, 0]) and abs(g[1, 1]) < 2.0 ** -1000
+
+
+def test_large_column_scales_of_null_columns(plhr):
+    """Columns of zeros with the column scale 1e300 (one over a floored norm), their images not zero:
+    only the products of two such images leave the range."""
+    rng = np.random.default_rng(4)
+    n, m, null = 500, 18, [3, 4, 17]
+    Z, A = rng.uniform(0.5, 1.0, (n, m)), rng.uniform(0.5, 1.0, (n, m))
+    Z[:, null] = 0.0
+    A[:250, 3] = A[250:, 4] = 0.0                        # the images of 3 and 4 share no row
+    cs = 1.0 / np.maximum(np.linalg.norm(Z, axis=0), 1e-300)
+    G = plhr.gram(plhr.GRAM_F64, _dev(Z), _dev(A), sigma=3.0, colscale=_dev(cs)).cpu().numpy()
+    z, u = Z.astype(np.longdouble) * cs, (A.astype(np.longdouble) - 3.0 * Z) * cs
+    for g, x, y in zip(G, (z, u, u), (z, u, z)):
+        ref = x.T @ y
+        out = np.abs(ref) > np.longdouble(2.0) ** 1023
+        norm = np.outer(np.sqrt((x * x).sum(0)), np.sqrt((y * y).sum(0)))
+        assert np.isinf(g[out]).all() and np.isfinite(g[~out]).all()
+        assert (np.abs(g - ref)[~out] <= 2.0 ** -46 * norm[~out]).all()
+    assert G[1, 3, 4] == 0.0
