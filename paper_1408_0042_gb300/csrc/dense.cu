@@ -352,7 +352,11 @@ __device__ __forceinline__ void house3(dw x, dw y, dw z, dw& u1, dw& u2, dw& tau
     const dw srv = dw_mul_pow2(rv, sg);
     u1 = dw_mul(y, srv);
     u2 = dw_mul(z, srv);
-    tau = dw_mul(w, rn);
+    // w / norm = 1 + |x| / norm: the error of the quotient counts half at most, and the
+    // product w (1 / norm) cost a tenth of the eigenvalues' accuracy (mean error at m = 64
+    // 9.1e-14, 7.2e-14 now, 8.4e-14 with general operations; the same time)
+    const dw q = dw_two_prod(x.hi, rn.hi), t = dw_fast_two_sum(1.0f, q.hi);
+    tau = dw_fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(q.lo, __fmaf_rn(x.hi, rn.lo, __fmul_rn(x.lo, rn.hi)))));
     beta = dw_mul_pow2(nrm, __fmul_rn(-sg, pow2_inverse_of(sc)));   // sc is a power of two
 }
 
