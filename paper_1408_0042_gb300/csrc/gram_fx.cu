@@ -66,7 +66,7 @@
 //
 // Measured on GB300 on trial bases of a Laplacian: m = 36, 262,144 rows 370 us a call
 // (FP64 multiply-adds 2.64 ms, bound by the FP64 pipe); m = 64, 2,097,152 rows
-// 2.56 ms (double-word multiply-adds on the FP32 pipes 9.45 ms).
+// 2.61 ms a call, 2.53 of the kernel (double-word multiply-adds on the FP32 pipes 9.45 ms).
 #include "blockops.h"
 #include "tc.h"
 
